@@ -153,6 +153,9 @@ struct fld_handle {
     long long ncell = 0;
     LevelBufs<double> d64[MAX_LEVELS];
     LevelBufs<float> d32[MAX_LEVELS];
+    // FP64 V-cycle coefficients of 2D and 3D levels: slices of the two pools below, which
+    // hold the double-FP32 vectors and the FP32 pyramid in the mixed modes
+    Coef64 w64[MAX_LEVELS] = {};
     float* dfx[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // iterate (hi, lo), ping-pong
     float* dfb[2] = {nullptr, nullptr};                            // right-hand side (hi, lo)
     float* dfK[2] = {nullptr, nullptr};                            // coefficient K (hi, lo)
@@ -346,6 +349,66 @@ void choose_depth(fld_handle* h, double kmax) {
     }
 }
 
+// Levels whose FP64 V-cycle runs on stored coefficients: those above the single-block tail
+// or the coarsest level, in 2D and 3D.
+bool coef_level(const fld_handle* h, int l) {
+    const int end = h->tail_start >= 0 ? h->tail_start : h->nlev - 1;
+    return (l == 0 || l < end) && mg64_ok(h->lv[l]);
+}
+
+// The FP32 storage of a handle as two pools, sliced for either use: df_pool the eight
+// double-FP32 vectors, or the four coefficient arrays of level 0 in an FP64 solve; pool32 the
+// FP32 pyramid, or the coefficient arrays of the coarser levels (a quarter or less of level
+// 0's cells in all, so they take less room than the pyramid's four floats a cell).
+// A slice starts on 256 bytes.
+constexpr long long slice_floats(long long n) { return (n + 63) & ~63LL; }
+
+long long df_pool_floats(const fld_handle* h) { return 8 * slice_floats(h->ncell); }
+
+long long pool32_floats(const fld_handle* h) {
+    long long a = 0, b = 0;
+    for (int l = 0; l < h->nlev; ++l) {
+        a += 4 * slice_floats(h->lv[l].ncell);
+        if (l > 0 && coef_level(h, l)) b += 4 * slice_floats(2 * h->lv[l].ncell);
+    }
+    return std::max(a, b);
+}
+
+void slice_pools(fld_handle* h, float* df_pool, float* pool32) {
+    auto take = [](float*& at, long long n) {
+        float* q = at;
+        at += slice_floats(n);
+        return q;
+    };
+    const long long n0 = h->ncell;
+    float* p = df_pool;
+    for (int q = 0; q < 2; ++q) {
+        h->dfx[q][0] = take(p, n0);
+        h->dfx[q][1] = take(p, n0);
+        h->dfb[q] = take(p, n0);
+        h->dfK[q] = take(p, n0);
+    }
+    p = pool32;
+    for (int l = 0; l < h->nlev; ++l) {
+        const long long n = h->lv[l].ncell;
+        h->d32[l].x = take(p, n);
+        h->d32[l].b = take(p, n);
+        h->d32[l].K = take(p, n);
+        h->d32[l].tmp = take(p, n);
+    }
+    p = pool32;
+    for (int l = 0; l < h->nlev; ++l) {
+        h->w64[l] = Coef64{nullptr, nullptr, nullptr, nullptr};
+        if (!coef_level(h, l)) continue;
+        float*& at = l == 0 ? df_pool : p;
+        const long long n = 2 * h->lv[l].ncell;
+        h->w64[l].wx = (double*)take(at, n);
+        h->w64[l].wy = (double*)take(at, n);
+        h->w64[l].wz = (double*)take(at, n);
+        h->w64[l].inv = (double*)take(at, n);
+    }
+}
+
 template <typename T>
 fld_status dalloc(fld_handle* h, T** p, long long n) {
     void* q = nullptr;
@@ -414,6 +477,19 @@ void smooth(fld_handle* h, LevelBufs<T>& B, int l, int n, int fused, T*& cur, T*
         std::swap(cur, oth);
     }
     int left = n - fused;
+    if constexpr (sizeof(T) == 8) {
+        if (const Coef64& W = h->w64[l]; W.inv) {
+            const bool inplace = h->o.smoother != 1 && rb_half_supported<T>(L);
+            T* mid = inplace ? cur : oth;
+            for (; left > 0; --left) {
+                run(h, "rbhalf64", l, L.ncell, s,
+                    [&] { launch_half64(L, 0, cur, mid, B.b, W, s); });
+                run(h, "rbhalf64", l, L.ncell, s,
+                    [&] { launch_half64(L, 1, mid, cur, B.b, W, s); });
+            }
+            return;
+        }
+    }
     if (h->o.smoother != 1 && rb_half_supported<T>(L)) {
         const char* nm = f32 ? "rbhalf32" : "rbhalf64";
         for (; left > 0; --left) {
@@ -479,8 +555,14 @@ void vcycle(fld_handle* h, LevelBufs<T>* P, int l, cudaStream_t s) {
     T* oth = B.tmp;
     smooth<T>(h, B, l, nu1, f1, cur, oth, s);
     const Lvl& C = h->lv[l + 1];
-    run(h, f32 ? "resid_restrict32" : "resid_restrict64", l, L.ncell, s,
-        [&] { launch_resid_restrict<T>(L, C, cur, B.b, B.K, P[l + 1].b, bs, nu1 > 0, s); });
+    run(h, f32 ? "resid_restrict32" : "resid_restrict64", l, L.ncell, s, [&] {
+        if constexpr (sizeof(T) == 8) {
+            if (h->w64[l].inv)
+                return launch_restrict64(L, C, cur, B.b, B.K, h->w64[l], P[l + 1].b,
+                                         nu1 > 0 && !L.fm, s);
+        }
+        launch_resid_restrict<T>(L, C, cur, B.b, B.K, P[l + 1].b, bs, nu1 > 0, s);
+    });
     if (l + 1 < h->nlev - 1) cudaMemsetAsync(P[l + 1].x, 0, sizeof(T) * C.ncell, s);
     vcycle<T>(h, P, l + 1, s);
     run(h, f32 ? "prolong32" : "prolong64", l, L.ncell, s,
@@ -511,7 +593,12 @@ fld_status residual(fld_handle* h, const double* x, const float* e, double* xo, 
                     cudaStream_t s, double* rr, unsigned* err) {
     const Lvl& L = h->lv[0];
     int nparts = h->norm_blocks;
-    if (resid64z_ok(L, h->norm_blocks)) {
+    if (h->o.precision == FLD_PREC_FP64 && h->w64[0].inv) {
+        run(h, "resid64", 0, L.ncell, s, [&] {
+            nparts = launch_norm64(L, x, h->d64[0].b, h->d64[0].K, h->w64[0], h->partials,
+                                   h->norm_blocks, s);
+        });
+    } else if (resid64z_ok(L, h->norm_blocks)) {
         run(h, e ? "resid64x" : "resid64", 0, L.ncell, s, [&] {
             nparts = launch_resid64z(L, x, e, xo, h->d64[0].b, h->d64[0].K, r32, h->partials,
                                      h->norm_blocks, s);
@@ -700,7 +787,13 @@ fld_status diffuse_impl(fld_handle* h, double dt, const double* D, const double*
     });
     if (!direct) {
         if (mixed) restrict_pyramid<float>(h, h->d32, s);
-        else restrict_pyramid<double>(h, h->d64, s);
+        else {
+            restrict_pyramid<double>(h, h->d64, s);
+            for (int l = 0; l < h->nlev; ++l)
+                if (h->w64[l].inv)
+                    run(h, "coef64", l, h->lv[l].ncell, s,
+                        [&] { launch_coef64(h->lv[l], h->d64[l].K, h->w64[l], s); });
+        }
     }
     run(h, "sumsq", 0, L0.ncell, s,
         [&] { launch_sumsq(L0.ncell, h->d64[0].b, h->partials, h->norm_blocks, s); });
@@ -925,19 +1018,10 @@ fld_status fld_create(fld_handle** out, const fld_grid* g, const fld_opts* o) {
         rc = rc ? rc : dalloc(h, &h->d64[l].K, n);
         rc = rc ? rc : dalloc(h, &h->d64[l].tmp, n);
     }
-    for (int l = 0; l < h->nlev && !rc; ++l) {
-        const long long n = h->lv[l].ncell;
-        rc = rc ? rc : dalloc(h, &h->d32[l].x, n);
-        rc = rc ? rc : dalloc(h, &h->d32[l].b, n);
-        rc = rc ? rc : dalloc(h, &h->d32[l].K, n);
-        rc = rc ? rc : dalloc(h, &h->d32[l].tmp, n);
-    }
-    for (int q = 0; q < 2 && !rc; ++q) {
-        rc = rc ? rc : dalloc(h, &h->dfx[q][0], n0);
-        rc = rc ? rc : dalloc(h, &h->dfx[q][1], n0);
-        rc = rc ? rc : dalloc(h, &h->dfb[q], n0);
-        rc = rc ? rc : dalloc(h, &h->dfK[q], n0);
-    }
+    float *df_pool = nullptr, *pool32 = nullptr;
+    rc = rc ? rc : dalloc(h, &df_pool, df_pool_floats(h));
+    rc = rc ? rc : dalloc(h, &pool32, pool32_floats(h));
+    if (!rc) slice_pools(h, df_pool, pool32);
     rc = rc ? rc : dalloc(h, &h->Dscratch, n0);
     rc = rc ? rc : dalloc(h, &h->krscratch, n0);
     if (g->ndim == 1) rc = rc ? rc : dalloc(h, &h->triw, 12 * n0 + 1);
@@ -1342,19 +1426,10 @@ extern "C" fld_status fld_diffuse_static(const fld_grid* g, const fld_opts* o, d
         h.d64[l].K = (double*)take(8 * n);
         h.d64[l].tmp = (double*)take(8 * n);
     }
-    for (int l = 0; l < h.nlev; ++l) {
-        const long long n = h.lv[l].ncell;
-        h.d32[l].x = (float*)take(4 * n);
-        h.d32[l].b = (float*)take(4 * n);
-        h.d32[l].K = (float*)take(4 * n);
-        h.d32[l].tmp = (float*)take(4 * n);
-    }
-    for (int q = 0; q < 2; ++q) {
-        h.dfx[q][0] = (float*)take(4 * n0);
-        h.dfx[q][1] = (float*)take(4 * n0);
-        h.dfb[q] = (float*)take(4 * n0);
-        h.dfK[q] = (float*)take(4 * n0);
-    }
+    float* df_pool = (float*)take(4 * df_pool_floats(&h));
+    float* pool32 = (float*)take(4 * pool32_floats(&h));
+    if (!fits) return FLD_ERR_ARG;
+    slice_pools(&h, df_pool, pool32);
     h.norm_blocks = NORM_BLOCKS_PER_SM * num_sms();
     h.partials = (double*)take(24 * (size_t)h.norm_blocks);
     h.scal = (DevScalars*)take(sizeof(DevScalars));

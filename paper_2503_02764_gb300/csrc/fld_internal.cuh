@@ -290,6 +290,23 @@ template <typename T>
 size_t tail_smem_bytes(const Lvl* lv, int n);
 void prepare_vcycle_tail();
 
+// FP64 V-cycle on stored coefficients (k_mg64.cu): face weights towards the lower neighbour
+// along each axis and the inverse diagonal, formed once per level and solve.
+struct Coef64 {
+    double *wx, *wy, *wz, *inv;
+};
+bool mg64_ok(const Lvl& L);
+void launch_coef64(const Lvl& L, const double* K, const Coef64& W, cudaStream_t s);
+// one colour's relaxation, in place (xin == xout) or with the other colour copied
+void launch_half64(const Lvl& L, int color, const double* xin, double* xout, const double* b,
+                   const Coef64& W, cudaStream_t s);
+// partial sums of ||b - A x||^2; returns their number (<= nblocks)
+int launch_norm64(const Lvl& L, const double* x, const double* b, const double* K,
+                  const Coef64& W, double* partials, int nblocks, cudaStream_t s);
+void launch_restrict64(const Lvl& F, const Lvl& C, const double* x, const double* b,
+                       const double* K, const Coef64& W, double* bc, bool red_only,
+                       cudaStream_t s);
+
 // 3D transfers when every axis halves exactly (one thread per coarse cell).
 bool transfer3_ok(const Lvl& F, const Lvl& C);
 // red_only: the level was just smoothed by a red-black sweep (black last), so only the

@@ -274,8 +274,10 @@ __global__ void k_resid_restrict(Lvl F, Lvl C, const T* __restrict__ x, const T*
 template <typename T>
 void launch_resid_restrict(const Lvl& F, const Lvl& C, const T* x, const T* b, const T* K, T* bc,
                            int block, bool red_only, cudaStream_t s) {
-    if (transfer3_ok(F, C) && !F.fm)
-        return launch_resid_restrict3<T>(F, C, x, b, K, bc, red_only, s);
+    // (FP64 3D levels run on stored coefficients, k_mg64.cu)
+    if constexpr (sizeof(T) == 4)
+        if (transfer3_ok(F, C) && !F.fm)
+            return launch_resid_restrict3<T>(F, C, x, b, K, bc, red_only, s);
     k_resid_restrict<T><<<grid_for(C.ncell, block), block, 0, s>>>(F, C, x, b, K, bc);
 }
 
