@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "fld_internal.cuh"
+#include "fld_line.cuh"
 
 using namespace fld;
 
@@ -37,6 +38,7 @@ struct DevScalars {       // read back together after each cycle
     double energy[2];     // diagnostics: total energy before and after a call
     double drift;         // recursive residual: sum of the squared scaled rounding bound
     double amax;          //   and the largest absolute row sum of the level-0 operator
+    LineOut line;         // the one-launch 1D solve's result
 };
 
 std::atomic<long long> g_launches{0};
@@ -769,8 +771,55 @@ fld_status diffuse_df(fld_handle* h, double* E, double bsum, fld_stats* st, cuda
     return rel <= h->o.tol ? FLD_OK : FLD_ERR_NOT_CONVERGED;
 }
 
+// A line (1D grid) short enough for one launch: the direct solve of D's system, or with `step`
+// the whole substep, then one read-back. A cell that fails the domain check ends it before
+// anything is written; a solve that diverged ends it before the exchange.
+bool line_direct(const fld_handle* h) {
+    return h->g.ndim == 1 && h->o.direct1d && h->triw && line_ok(h->lv[0]);
+}
+
+LineArgs line_args(const fld_handle* h, double dt, const double* E_bc, double* E) {
+    LineArgs a{};
+    a.L = h->lv[0];
+    for (int q = 0; q < 6; ++q) a.bo.off[q] = h->bc_off[q];
+    a.Ebc = E_bc;
+    a.E = E;
+    a.kscale = dt / (h->g.h[0] * h->g.h[0]);
+    a.tol = h->o.tol;
+    a.max_cycles = h->o.max_cycles;
+    a.one = 1.0;
+    return a;
+}
+
+fld_status line_run(fld_handle* h, const LineArgs& a, bool step, fld_stats* st, cudaStream_t s) {
+    run(h, step ? "line_step" : "line_solve", 0, h->ncell, s,
+        [&] { launch_line(a, step, &h->scal->line, &h->scal->err, s); });
+    FLD_CK(cudaGetLastError());
+    double sum;
+    unsigned err;
+    const fld_status rc = read_scalars(h, s, &sum, &err);
+    if (rc != FLD_OK) return rc;
+    if (err) cudaMemsetAsync(&h->scal->err, 0, sizeof(unsigned), s);
+    const LineOut& o = h->hscal->line;
+    if (o.cyc == 0) return FLD_ERR_DOMAIN;
+    if (st) {
+        memset(st, 0, sizeof(*st));
+        for (int q = 0; q <= o.cyc && q < 64; ++q) st->resid_hist[q] = o.hist[q];
+        st->levels = 1;
+        st->cycles = o.cyc;
+        st->rel_resid = o.rel;
+    }
+    if (err || !std::isfinite(o.rel)) return FLD_ERR_DOMAIN;
+    return o.rel <= h->o.tol ? FLD_OK : FLD_ERR_NOT_CONVERGED;
+}
+
 fld_status diffuse_impl(fld_handle* h, double dt, const double* D, const double* E_bc, double* E,
                         fld_stats* st, cudaStream_t s) {
+    if (line_direct(h)) {
+        LineArgs a = line_args(h, dt, E_bc, E);
+        a.D = D;
+        return line_run(h, a, false, st, s);
+    }
     const Lvl& L0 = h->lv[0];
     const bool dfmode = h->o.precision == FLD_PREC_MIXED_DF;
     const bool mixed = h->o.precision == FLD_PREC_MIXED || dfmode;
@@ -1041,6 +1090,7 @@ fld_status fld_create(fld_handle** out, const fld_grid* g, const fld_opts* o) {
     if (!rc) {
         prepare_rb_sweep();
         prepare_vcycle_tail();
+        prepare_line();
         debug_attach_all();
     }
     if (!rc && cudaDeviceSynchronize() != cudaSuccess) rc = FLD_ERR_CUDA;
@@ -1239,6 +1289,21 @@ fld_status fld_step(fld_handle* h, const fld_consts* k, const fld_opacity* op, d
     cudaStream_t s = (cudaStream_t)stream;
     const bool en = want(h, stats, FLD_DIAG_ENERGY), tm = want(h, stats, FLD_DIAG_TIMES);
     const double cv = k->R_gas / (k->gamma - 1.0);
+    // one launch for a whole 1D substep in FP64 arithmetic; the diagnostics and the
+    // double-FP32 limiter and exchange take the separate parts
+    if (!en && !tm && line_direct(h) && h->o.precision != FLD_PREC_MIXED_DF && !h->o.limiter_df) {
+        LineArgs a = line_args(h, dt, E_bc, E);
+        a.op = to_op(op);
+        a.rho = rho;
+        a.T = T;
+        a.inv12h = 1.0 / (12.0 * h->g.h[0]);
+        a.c = k->c;
+        a.dtc = dt * k->c;
+        a.a_r = k->a_r;
+        a.cv = cv;
+        a.mode = h->o.limiter;
+        return line_run(h, a, true, stats, s);
+    }
     if (tm) FLD_CK(cudaEventRecord(h->tev[0], s));
     if (en) energy_sum(h, rho, T, E, cv, 0, s);
     // the limiter freezes kappa rho at (rho, T^n) for the exchange (one opacity evaluation
