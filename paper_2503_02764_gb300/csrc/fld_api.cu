@@ -13,6 +13,7 @@
 
 #include "fld_internal.cuh"
 #include "fld_line.cuh"
+#include "fld_wave1d.cuh"
 
 using namespace fld;
 
@@ -38,7 +39,7 @@ struct DevScalars {       // read back together after each cycle
     double energy[2];     // diagnostics: total energy before and after a call
     double drift;         // recursive residual: sum of the squared scaled rounding bound
     double amax;          //   and the largest absolute row sum of the level-0 operator
-    LineOut line;         // the one-launch 1D solve's result
+    LineOut line[2];      // results of the one-launch 1D solve (two stages of a wave step)
 };
 
 std::atomic<long long> g_launches{0};
@@ -791,17 +792,48 @@ LineArgs line_args(const fld_handle* h, double dt, const double* E_bc, double* E
     return a;
 }
 
-fld_status line_run(fld_handle* h, const LineArgs& a, bool step, fld_stats* st, cudaStream_t s) {
-    run(h, step ? "line_step" : "line_solve", 0, h->ncell, s,
-        [&] { launch_line(a, step, &h->scal->line, &h->scal->err, s); });
+// the same with the limiter and the exchange, in FP64 arithmetic
+bool line_step_ok(const fld_handle* h) {
+    return line_direct(h) && h->o.precision != FLD_PREC_MIXED_DF && !h->o.limiter_df;
+}
+
+void line_physics(const fld_handle* h, const fld_consts* k, const fld_opacity* op, double dt,
+                  LineArgs& a) {
+    a.op = to_op(op);
+    a.inv12h = 1.0 / (12.0 * h->g.h[0]);
+    a.c = k->c;
+    a.dtc = dt * k->c;
+    a.a_r = k->a_r;
+    a.cv = k->R_gas / (k->gamma - 1.0);
+    a.mode = h->o.limiter;
+}
+
+fld_status line_launch(fld_handle* h, const LineArgs& a, int kind, int slot, cudaStream_t s) {
+    run(h, kind == LINE_SOLVE ? "line_solve" : "line_step", 0, h->ncell, s,
+        [&] { launch_line(a, kind, &h->scal->line[slot], &h->scal->err, s); });
     FLD_CK(cudaGetLastError());
+    return FLD_OK;
+}
+
+// The read-back of `slots` launches; the statistics are the last one's. A wave step's stages
+// are judged by their own outcome: a flag that an explicit evaluation raised after them stays
+// for the next step's first stage.
+fld_status line_collect(fld_handle* h, bool wave, int slots, fld_stats* st, cudaStream_t s) {
     double sum;
     unsigned err;
     const fld_status rc = read_scalars(h, s, &sum, &err);
     if (rc != FLD_OK) return rc;
-    if (err) cudaMemsetAsync(&h->scal->err, 0, sizeof(unsigned), s);
-    const LineOut& o = h->hscal->line;
-    if (o.cyc == 0) return FLD_ERR_DOMAIN;
+    bool conv = true, failed = !wave && err;
+    bool none = false;               // a solve that never ran
+    for (int q = 0; q < slots; ++q) {
+        const LineOut& o = h->hscal->line[q];
+        none = none || o.cyc == 0;
+        failed = failed || none || (wave && o.failed) || !std::isfinite(o.rel);
+        conv = conv && o.rel <= h->o.tol;
+    }
+    if (failed && err) cudaMemsetAsync(&h->scal->err, 0, sizeof(unsigned), s);
+    if (none) return FLD_ERR_DOMAIN;
+    const LineOut& o = h->hscal->line[slots - 1];
     if (st) {
         memset(st, 0, sizeof(*st));
         for (int q = 0; q <= o.cyc && q < 64; ++q) st->resid_hist[q] = o.hist[q];
@@ -809,8 +841,12 @@ fld_status line_run(fld_handle* h, const LineArgs& a, bool step, fld_stats* st, 
         st->cycles = o.cyc;
         st->rel_resid = o.rel;
     }
-    if (err || !std::isfinite(o.rel)) return FLD_ERR_DOMAIN;
-    return o.rel <= h->o.tol ? FLD_OK : FLD_ERR_NOT_CONVERGED;
+    return failed ? FLD_ERR_DOMAIN : conv ? FLD_OK : FLD_ERR_NOT_CONVERGED;
+}
+
+fld_status line_run(fld_handle* h, const LineArgs& a, int kind, fld_stats* st, cudaStream_t s) {
+    const fld_status rc = line_launch(h, a, kind, 0, s);
+    return rc != FLD_OK ? rc : line_collect(h, false, 1, st, s);
 }
 
 fld_status diffuse_impl(fld_handle* h, double dt, const double* D, const double* E_bc, double* E,
@@ -818,7 +854,7 @@ fld_status diffuse_impl(fld_handle* h, double dt, const double* D, const double*
     if (line_direct(h)) {
         LineArgs a = line_args(h, dt, E_bc, E);
         a.D = D;
-        return line_run(h, a, false, st, s);
+        return line_run(h, a, LINE_SOLVE, st, s);
     }
     const Lvl& L0 = h->lv[0];
     const bool dfmode = h->o.precision == FLD_PREC_MIXED_DF;
@@ -1291,18 +1327,12 @@ fld_status fld_step(fld_handle* h, const fld_consts* k, const fld_opacity* op, d
     const double cv = k->R_gas / (k->gamma - 1.0);
     // one launch for a whole 1D substep in FP64 arithmetic; the diagnostics and the
     // double-FP32 limiter and exchange take the separate parts
-    if (!en && !tm && line_direct(h) && h->o.precision != FLD_PREC_MIXED_DF && !h->o.limiter_df) {
+    if (!en && !tm && line_step_ok(h)) {
         LineArgs a = line_args(h, dt, E_bc, E);
-        a.op = to_op(op);
+        line_physics(h, k, op, dt, a);
         a.rho = rho;
         a.T = T;
-        a.inv12h = 1.0 / (12.0 * h->g.h[0]);
-        a.c = k->c;
-        a.dtc = dt * k->c;
-        a.a_r = k->a_r;
-        a.cv = cv;
-        a.mode = h->o.limiter;
-        return line_run(h, a, true, stats, s);
+        return line_run(h, a, LINE_STEP, stats, s);
     }
     if (tm) FLD_CK(cudaEventRecord(h->tev[0], s));
     if (en) energy_sum(h, rho, T, E, cv, 0, s);
@@ -1328,6 +1358,36 @@ fld_status fld_step(fld_handle* h, const fld_consts* k, const fld_opacity* op, d
 }  // extern "C"
 
 long long fld::fld_handle_cells(const fld_handle* h) { return h ? h->ncell : 0; }
+
+// ---- the wave step's implicit stage (fld_wave1d_api.cu)
+bool fld::fld_line_wave_ok(const fld_handle* h) { return line_step_ok(h) && !h->o.diag; }
+
+bool fld::fld_physics_ok(const fld_consts* k, const fld_opacity* op) {
+    return consts_ok(k) && op_ok(op);
+}
+
+fld_status fld::fld_line_wave(fld_handle* h, const fld_consts* k, const fld_opacity* op,
+                              double tau, const LineWave& w, const double* E_bc, int slot,
+                              cudaStream_t s) {
+    if (!(tau > 0) || !std::isfinite(tau)) return FLD_ERR_ARG;
+    LineArgs a = line_args(h, tau, E_bc, nullptr);
+    line_physics(h, k, op, tau, a);
+    a.rho = w.Uin;
+    a.E = const_cast<double*>(w.Uin) + 7 * h->ncell;      // read only in this kind
+    a.T = w.T;
+    a.w = w;
+    return line_launch(h, a, LINE_WAVE, slot, s);
+}
+
+fld_status fld::fld_line_collect(fld_handle* h, int slots, fld_stats* st, cudaStream_t s) {
+    return line_collect(h, true, slots, st, s);
+}
+
+const unsigned* fld::fld_line_failed(fld_handle* h, int slot) { return &h->scal->line[slot].failed; }
+
+unsigned* fld::fld_handle_err(fld_handle* h) { return &h->scal->err; }
+
+Opacity fld::fld_to_opacity(const fld_opacity* op) { return to_op(op); }
 
 extern "C" {
 

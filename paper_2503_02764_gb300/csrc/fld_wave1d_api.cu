@@ -16,12 +16,10 @@ struct fld_wave1d {
     Wave1dDev dev;
     fld_handle* h = nullptr;
     std::vector<void*> allocs;
-    double *A = nullptr, *B = nullptr, *Fi = nullptr;
-    double *rho = nullptr, *vx = nullptr, *T = nullptr, *T0 = nullptr, *E = nullptr;
-    double *fr = nullptr, *vfr = nullptr, *pt = nullptr, *ebc = nullptr;
+    double *A = nullptr, *B = nullptr;
+    double *rho = nullptr, *T = nullptr, *T0 = nullptr, *E = nullptr, *ebc = nullptr;
     // ARS3 IMEX stages: explicit right-hand sides, predictor, implicit increments (e, E)
-    double *L1 = nullptr, *L2 = nullptr, *L3 = nullptr, *Pp = nullptr, *G2 = nullptr,
-           *G3 = nullptr;
+    double *L1 = nullptr, *L2 = nullptr, *Pp = nullptr, *G2 = nullptr, *G3 = nullptr;
     unsigned long long* smax = nullptr;
 };
 
@@ -71,62 +69,88 @@ fld_consts step_consts(const fld_wave1d* w) {
     return k;
 }
 
+// what every explicit evaluation of a step shares
+W1Stage stage_of(fld_wave1d* w, double dt) {
+    W1Stage g{};
+    g.rad = w->p.radiation;
+    g.op = fld_to_opacity(&w->p.opacity);
+    g.c = w->p.consts.c;
+    g.E_right = w->p.E_right;
+    g.mode = w->p.opts.limiter;
+    g.err = fld_handle_err(w->h);
+    g.dt = dt;
+    return g;
+}
+
+fld_status advance(fld_wave1d* w, const W1Stage& g, cudaStream_t s) {
+    launch_w1_advance(w->dev, g, s);
+    note_launches(1);
+    return cudaGetLastError() == cudaSuccess ? FLD_OK : FLD_ERR_CUDA;
+}
+
 // one Runge-Kutta stage: Uout = a U0 + b (Uin + dt L(Uin)) at time t_in, driven at t_out
 fld_status stage(fld_wave1d* w, const double* U0, const double* Uin, double* Uout, double a,
                  double b, double dt, double t_in, double t_out, cudaStream_t s) {
-    const Wave1dDev& P = w->dev;
-    const fld_consts k = step_consts(w);
-    if (w->p.radiation) {
-        launch_w1_prim(P, Uin, w->rho, w->vx, w->T, nullptr, w->E, s);
-        fld_status rc = fld_coupling(w->h, &k, &w->p.opacity, w->E, w->rho, w->T, w->ebc, w->vx,
-                                     nullptr, w->fr, nullptr, w->vfr, w->pt, s);
-        if (rc != FLD_OK) return rc;
-    }
-    launch_w1_iface(P, Uin, t_in, w->Fi, s);
-    launch_w1_stage(P, U0, Uin, Uout, w->Fi, w->fr, w->vfr, w->pt, a, b, dt, t_out, s);
-    note_launches(3);
-    return cudaGetLastError() == cudaSuccess ? FLD_OK : FLD_ERR_CUDA;
+    W1Stage g = stage_of(w, dt);
+    g.ssp = 1;
+    g.U0 = U0;
+    g.Uin = Uin;
+    g.Uout = Uout;
+    g.a = a;
+    g.b = b;
+    g.t_in = t_in;
+    g.t_out = t_out;
+    return advance(w, g, s);
 }
 
-// the explicit right-hand side L(Uin) at time t (hyperbolic fluxes with the driven left
-// ghosts at t, plus the coupling terms)
-fld_status explicit_rhs(fld_wave1d* w, const double* Uin, double t, double* Lout,
-                        cudaStream_t s) {
-    const Wave1dDev& P = w->dev;
-    const fld_consts k = step_consts(w);
-    if (w->p.radiation) {
-        launch_w1_prim(P, Uin, w->rho, w->vx, w->T, nullptr, w->E, s);
-        fld_status rc = fld_coupling(w->h, &k, &w->p.opacity, w->E, w->rho, w->T, w->ebc, w->vx,
-                                     nullptr, w->fr, nullptr, w->vfr, w->pt, s);
-        if (rc != FLD_OK) return rc;
-    }
-    launch_w1_iface(P, Uin, t, w->Fi, s);
-    launch_w1_rhs(P, w->Fi, w->fr, w->vfr, w->pt, Lout, s);
-    note_launches(3);
-    return cudaGetLastError() == cudaSuccess ? FLD_OK : FLD_ERR_CUDA;
-}
-
-// an implicit stage: Uout = the FLD substep over tau from the predictor Pin (the gas energy
-// takes the exchange's change of T_g; driven cells at t_drive), G its increment / tau
+// An implicit stage: Uout = the FLD substep over tau from the predictor Pin (the gas energy
+// takes the exchange's change of T_g; driven cells at t_drive), G (nullable) its increment / tau.
+// In one launch where the line allows it: its outcome is then read back with the step's
+// (fld_line_collect), and what follows it is held back by the domain flag.
 fld_status implicit_stage(fld_wave1d* w, const double* Pin, double* Uout, double* G, double tau,
-                          double t_drive, fld_stats* stats, cudaStream_t s) {
+                          double t_drive, int slot, fld_stats* stats, cudaStream_t s) {
     const long long n = w->p.n;
-    if (cudaMemcpyAsync(Uout, Pin, sizeof(double) * 8 * n, cudaMemcpyDeviceToDevice, s) !=
-        cudaSuccess)
+    const fld_consts k = step_consts(w);
+    if (w->p.radiation && fld_line_wave_ok(w->h)) {
+        LineWave v{};
+        v.P = w->dev;
+        v.Uin = Pin;
+        v.Uout = Uout;
+        v.T = w->T;
+        v.G = G;
+        v.inv_tau = 1.0 / tau;
+        v.t_drive = t_drive;
+        return fld_line_wave(w->h, &k, &w->p.opacity, tau, v, w->ebc, slot, s);
+    }
+    if (Uout != Pin && cudaMemcpyAsync(Uout, Pin, sizeof(double) * 8 * n,
+                                       cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return FLD_ERR_CUDA;
-    if (!w->p.radiation)   // no implicit terms: the stage value is the predictor
+    if (!w->p.radiation) {   // no implicit terms: the stage value is the predictor
+        if (!G) return FLD_OK;
         return cudaMemsetAsync(G, 0, sizeof(double) * 2 * n, s) == cudaSuccess ? FLD_OK
                                                                                : FLD_ERR_CUDA;
-    launch_w1_prim(w->dev, Uout, w->rho, w->vx, w->T, w->T0, w->E, s);
+    }
+    launch_w1_prim(w->dev, Uout, w->rho, w->T, w->T0, w->E, s);
     note_launches(1);
-    const fld_consts k = step_consts(w);
     const fld_status rc = fld_step(w->h, &k, &w->p.opacity, tau, w->rho, w->T, w->E, w->ebc,
                                    stats, s);
     if (rc != FLD_OK && rc != FLD_ERR_NOT_CONVERGED) return rc;
     launch_w1_post(w->dev, Uout, w->rho, w->T0, w->T, w->E, t_drive, s);
-    launch_w1_incr(w->dev, Uout, Pin, 1.0 / tau, G, s);
-    note_launches(2);
+    note_launches(1);
+    if (G) {
+        launch_w1_incr(w->dev, Uout, Pin, 1.0 / tau, G, s);
+        note_launches(1);
+    }
     return cudaGetLastError() == cudaSuccess ? rc : FLD_ERR_CUDA;
+}
+
+// The end of a step: the outcome of `slots` one-launch stages, or `rs` of the stages that were
+// read back as they ran.
+fld_status finish(fld_wave1d* w, int slots, fld_status rs, fld_stats* stats, cudaStream_t s) {
+    if (cudaGetLastError() != cudaSuccess) return FLD_ERR_CUDA;
+    if (w->p.radiation && fld_line_wave_ok(w->h))
+        return fld_line_collect(w->h, slots, stats, s);
+    return cudaStreamSynchronize(s) == cudaSuccess ? rs : FLD_ERR_CUDA;
 }
 
 // One ARS(2,3,3) step (Ascher, Ruuth and Spiteri 1997; the ARS3 of Sect. 3), gamma =
@@ -136,32 +160,47 @@ fld_status implicit_stage(fld_wave1d* w, const double* Pin, double* Uout, double
 // increments; predictors and stage values take the driving wave at their stage times.
 fld_status step_ars3(fld_wave1d* w, double* U, double t, double dt, fld_stats* stats,
                      cudaStream_t s) {
-    const double g = (3.0 + std::sqrt(3.0)) / 6.0;
-    const Wave1dDev& P = w->dev;
-    fld_status rc = explicit_rhs(w, U, t, w->L1, s);
+    const double ga = (3.0 + std::sqrt(3.0)) / 6.0;
+    const double t1 = t + ga * dt, t2 = t + (1.0 - ga) * dt;
+    W1Stage g = stage_of(w, dt);
+    g.U0 = U;
+    g.Uin = U;
+    g.Uout = w->Pp;
+    g.Lout = w->L1;
+    g.cn = ga;
+    g.t_in = t;
+    g.t_out = t1;
+    fld_status rc = advance(w, g, s);
     if (rc != FLD_OK) return rc;
-    launch_w1_comb(P, U, w->L1, nullptr, nullptr, g, 0.0, 0.0, nullptr, nullptr, 0.0, 0.0, dt,
-                   w->Pp, t + g * dt, s);
-    note_launches(1);
-    fld_status rs = implicit_stage(w, w->Pp, w->A, w->G2, g * dt, t + g * dt, stats, s);
+    fld_status rs = implicit_stage(w, w->Pp, w->A, w->G2, ga * dt, t1, 0, stats, s);
     if (rs != FLD_OK && rs != FLD_ERR_NOT_CONVERGED) return rs;
-    rc = explicit_rhs(w, w->A, t + g * dt, w->L2, s);
+    g.Uin = w->A;
+    g.La = w->L1;
+    g.ca = ga - 1.0;
+    g.cn = 2.0 * (1.0 - ga);
+    g.Lout = w->L2;
+    g.G2 = w->G2;
+    g.d2 = 1.0 - 2.0 * ga;
+    g.t_in = t1;
+    g.t_out = t2;
+    rc = advance(w, g, s);
     if (rc != FLD_OK) return rc;
-    launch_w1_comb(P, U, w->L1, w->L2, nullptr, g - 1.0, 2.0 * (1.0 - g), 0.0, w->G2, nullptr,
-                   1.0 - 2.0 * g, 0.0, dt, w->Pp, t + (1.0 - g) * dt, s);
-    note_launches(1);
-    const fld_status rs3 = implicit_stage(w, w->Pp, w->B, w->G3, g * dt, t + (1.0 - g) * dt,
-                                          stats, s);
+    const fld_status rs3 = implicit_stage(w, w->Pp, w->B, w->G3, ga * dt, t2, 1, stats, s);
     if (rs3 != FLD_OK && rs3 != FLD_ERR_NOT_CONVERGED) return rs3;
     if (rs3 != FLD_OK) rs = rs3;
-    rc = explicit_rhs(w, w->B, t + (1.0 - g) * dt, w->L3, s);
-    if (rc != FLD_OK) return rc;
-    launch_w1_comb(P, U, nullptr, w->L2, w->L3, 0.0, 0.5, 0.5, w->G2, w->G3, 0.5, 0.5, dt, U,
-                   t + dt, s);
-    note_launches(1);
-    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
-        return FLD_ERR_CUDA;
-    return rs;
+    g.Uin = w->B;
+    g.Uout = U;
+    g.Lout = nullptr;
+    g.La = nullptr;
+    g.Lb = w->L2;
+    g.cb = g.cn = g.d2 = g.d3 = 0.5;
+    g.G3 = w->G3;
+    g.t_in = t2;
+    g.t_out = t + dt;
+    // a failed stage leaves U as it was (elsewhere the failure was read back above)
+    if (w->p.radiation && fld_line_wave_ok(w->h)) g.gate = fld_line_failed(w->h, 1);
+    rc = advance(w, g, s);
+    return rc != FLD_OK ? rc : finish(w, 2, rs, stats, s);
 }
 
 }  // namespace
@@ -204,13 +243,11 @@ fld_status fld_wave1d_create(fld_wave1d** out, const fld_wave1d_params* p) {
         return rc;
     }
     const long long n = p->n;
-    bool ok = dal(w, &w->A, 8 * n) && dal(w, &w->B, 8 * n) && dal(w, &w->Fi, 8 * (n + 1)) &&
-              dal(w, &w->rho, n) && dal(w, &w->vx, n) && dal(w, &w->T, n) && dal(w, &w->T0, n) &&
-              dal(w, &w->E, n) && dal(w, &w->fr, n) && dal(w, &w->vfr, n) && dal(w, &w->pt, n) &&
-              dal(w, &w->ebc, 1);
+    bool ok = dal(w, &w->A, 8 * n) && dal(w, &w->B, 8 * n) && dal(w, &w->rho, n) &&
+              dal(w, &w->T, n) && dal(w, &w->T0, n) && dal(w, &w->E, n) && dal(w, &w->ebc, 1);
     if (ok && p->scheme == 1)
-        ok = dal(w, &w->L1, 8 * n) && dal(w, &w->L2, 8 * n) && dal(w, &w->L3, 8 * n) &&
-             dal(w, &w->Pp, 8 * n) && dal(w, &w->G2, 2 * n) && dal(w, &w->G3, 2 * n);
+        ok = dal(w, &w->L1, 8 * n) && dal(w, &w->L2, 8 * n) && dal(w, &w->Pp, 8 * n) &&
+             dal(w, &w->G2, 2 * n) && dal(w, &w->G3, 2 * n);
     double* sm = nullptr;
     ok = ok && dal(w, &sm, 1);
     w->smax = (unsigned long long*)sm;
@@ -218,11 +255,7 @@ fld_status fld_wave1d_create(fld_wave1d** out, const fld_wave1d_params* p) {
         destroy(w);
         return FLD_ERR_NOMEM;
     }
-    // the coupling sources stay zero without radiation
-    if (cudaMemset(w->fr, 0, sizeof(double) * n) != cudaSuccess ||
-        cudaMemset(w->vfr, 0, sizeof(double) * n) != cudaSuccess ||
-        cudaMemset(w->pt, 0, sizeof(double) * n) != cudaSuccess ||
-        cudaMemcpy(w->ebc, &p->E_right, sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (cudaMemcpy(w->ebc, &p->E_right, sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) {
         destroy(w);
         return FLD_ERR_CUDA;
     }
@@ -260,6 +293,8 @@ fld_status fld_wave1d_step(fld_wave1d* w, double* U, double t, double dt, fld_st
                            void* stream) {
     if (!w || !U || !finite_pos(dt) || !std::isfinite(t)) return FLD_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    const fld_consts k = step_consts(w);
+    if (w->p.radiation && !fld_physics_ok(&k, &w->p.opacity)) return FLD_ERR_ARG;
     if (w->p.scheme == 1) return step_ars3(w, U, t, dt, stats, s);
     // SSP-RK3: U1 = U + dt L(U); U2 = 3/4 U + 1/4 (U1 + dt L(U1));
     //          U3 = 1/3 U + 2/3 (U2 + dt L(U2)), written over U
@@ -268,22 +303,11 @@ fld_status fld_wave1d_step(fld_wave1d* w, double* U, double t, double dt, fld_st
     if (rc == FLD_OK)
         rc = stage(w, U, w->B, U, 1.0 / 3.0, 2.0 / 3.0, dt, t + 0.5 * dt, t + dt, s);
     if (rc != FLD_OK) return rc;
-    if (!w->p.radiation) {
-        if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
-            return FLD_ERR_CUDA;
-        return FLD_OK;
-    }
+    if (!w->p.radiation) return finish(w, 0, FLD_OK, stats, s);
     // FLD substep on (rho, T_g, E), then e += rho R_gas (T' - T) / (gamma - 1), E = E'
-    launch_w1_prim(w->dev, U, w->rho, w->vx, w->T, w->T0, w->E, s);
-    note_launches(1);
-    const fld_consts k = step_consts(w);
-    rc = fld_step(w->h, &k, &w->p.opacity, dt, w->rho, w->T, w->E, w->ebc, stats, s);
+    rc = implicit_stage(w, U, U, nullptr, dt, t + dt, 0, stats, s);
     if (rc != FLD_OK && rc != FLD_ERR_NOT_CONVERGED) return rc;
-    launch_w1_post(w->dev, U, w->rho, w->T0, w->T, w->E, t + dt, s);
-    note_launches(1);
-    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
-        return FLD_ERR_CUDA;
-    return rc;
+    return finish(w, 1, rc, stats, s);
 }
 
 }  // extern "C"

@@ -20,6 +20,7 @@
 
 #include "fld_device.cuh"
 #include "fld_line.cuh"
+#include "fld_wave1d.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -36,9 +37,10 @@ struct LineShared {
     double part[2];
 };
 
-template <bool STEP>
+template <int KIND>
 __global__ void __cluster_dims__(LINE_CS, 1, 1) __launch_bounds__(LINE_T)
 k_line(LineArgs g, int lg, LineOut* out, unsigned* err) {
+    constexpr bool STEP = KIND != LINE_SOLVE;
     extern __shared__ double arr[];
     __shared__ LineShared sh;
     cg::cluster_group cl = cg::this_cluster();
@@ -78,6 +80,12 @@ k_line(LineArgs g, int lg, LineOut* out, unsigned* err) {
     for (int q = threadIdx.x; q < mine; q += LINE_T) {
         const int i = first + q;
         double Dp, lm;
+        if (KIND == LINE_WAVE) {          // the gas temperature of the conserved state
+            double u[8], W[8];
+            for (int v = 0; v < 8; ++v) u[v] = g.w.Uin[(long long)v * n + i];
+            to_prim(u, g.w.P.Bx, g.w.P.gamma, W);
+            g.T[i] = W[6] / (W[0] * g.w.P.R_gas);
+        }
         if (STEP) {
             double kr = 0.0;
             if (!limiter_cell(g.L, ih, g.E, g.rho, g.T, g.Ebc, g.bo, g.op, g.c, g.mode, i, 0, 0, i,
@@ -107,6 +115,7 @@ k_line(LineArgs g, int lg, LineOut* out, unsigned* err) {
             atomicOr(err, ERRBIT_DOMAIN);
             out->cyc = 0;
             out->rel = 0.0;
+            out->failed = 1u;
         }
         return;
     }
@@ -227,6 +236,46 @@ k_line(LineArgs g, int lg, LineOut* out, unsigned* err) {
     if (rank == 0 && threadIdx.x == 0) {
         out->cyc = cyc;
         out->rel = rel;
+        out->failed = 0u;
+    }
+    if (KIND == LINE_WAVE) {
+        // nothing is written unless every cell of the line passes
+        double fail = isfinite(rel) ? 0.0 : 1.0;
+        for (int q = threadIdx.x; q < mine; q += LINE_T) {
+            const int i = first + q;
+            const double r = g.rho[i], kr = KR[q];
+            double t = g.T[i], er = X[q];
+            if (pos_finite(kr) && pos_finite(r) && pos_finite(t) && pos_finite(er))
+                exchange_cell_kr(r, kr, t, er, g.dtc, g.a_r, g.cv, g.one);
+            else
+                fail = 1.0;
+            KR[q] = t - g.T[i];
+            X[q] = er;
+        }
+        if (csum(fail) > 0.0) {
+            if (rank == 0 && threadIdx.x == 0) out->failed = 1u;
+            return;
+        }
+        const Wave1dDev& P = g.w.P;
+        for (int q = threadIdx.x; q < mine; q += LINE_T) {
+            const int i = first + q;
+            double u[8];
+            for (int v = 0; v < 8; ++v) u[v] = g.w.Uin[(long long)v * n + i];
+            const double e0 = u[6], E0 = u[7];
+            u[6] += u[0] * P.R_gas * KR[q] / (P.gamma - 1.0);
+            u[7] = X[q];
+            if (i < P.nd) {
+                double W[8];
+                drive_prim(P, (i + 0.5) * P.dx, g.w.t_drive, W);
+                to_cons(W, P.Bx, P.gamma, u);
+            }
+            for (int v = 0; v < 8; ++v) g.w.Uout[(long long)v * n + i] = u[v];
+            if (g.w.G) {
+                g.w.G[i] = (u[6] - e0) * g.w.inv_tau;
+                g.w.G[n + i] = (u[7] - E0) * g.w.inv_tau;
+            }
+        }
+        return;                                    // the sum above was the last remote read
     }
     const bool ex = STEP && isfinite(rel);         // a diverged solve ends before the exchange
     for (int q = threadIdx.x; q < mine; q += LINE_T) {
@@ -261,14 +310,17 @@ bool line_ok(const Lvl& L) { return L.ndim == 1 && L.n[0] <= LINE_CELLS; }
 
 void prepare_line() {
     const int most = (int)line_smem(line_lg(LINE_CELLS));
-    cudaFuncSetAttribute(k_line<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    cudaFuncSetAttribute(k_line<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(k_line<LINE_SOLVE>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(k_line<LINE_STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(k_line<LINE_WAVE>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
-void launch_line(const LineArgs& g, bool step, LineOut* out, unsigned* err, cudaStream_t s) {
+void launch_line(const LineArgs& g, int kind, LineOut* out, unsigned* err, cudaStream_t s) {
     const int lg = line_lg(g.L.n[0]);
-    if (step) k_line<true><<<LINE_CS, LINE_T, line_smem(lg), s>>>(g, lg, out, err);
-    else k_line<false><<<LINE_CS, LINE_T, line_smem(lg), s>>>(g, lg, out, err);
+    const size_t sm = line_smem(lg);
+    if (kind == LINE_STEP) k_line<LINE_STEP><<<LINE_CS, LINE_T, sm, s>>>(g, lg, out, err);
+    else if (kind == LINE_WAVE) k_line<LINE_WAVE><<<LINE_CS, LINE_T, sm, s>>>(g, lg, out, err);
+    else k_line<LINE_SOLVE><<<LINE_CS, LINE_T, sm, s>>>(g, lg, out, err);
 }
 
 }  // namespace fld

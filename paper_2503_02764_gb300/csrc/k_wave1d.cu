@@ -13,82 +13,21 @@ namespace {
 
 constexpr int W1_THREADS = 256;
 
-// conservative <-> primitive (rho, v_x, v_y, v_z, B_y, B_z, p, E)
-__device__ __forceinline__ void to_prim(const double* U, double Bx, double g, double* W) {
-    const double rho = U[0];
-    const double vx = U[1] / rho, vy = U[2] / rho, vz = U[3] / rho;
-    W[0] = rho;
-    W[1] = vx;
-    W[2] = vy;
-    W[3] = vz;
-    W[4] = U[4];
-    W[5] = U[5];
-    W[6] = (g - 1.0) * (U[6] - 0.5 * rho * (vx * vx + vy * vy + vz * vz) -
-                        0.5 * (Bx * Bx + U[4] * U[4] + U[5] * U[5]));
-    W[7] = U[7];
-}
-
-__device__ __forceinline__ void to_cons(const double* W, double Bx, double g, double* U) {
-    const double rho = W[0], vx = W[1], vy = W[2], vz = W[3];
-    U[0] = rho;
-    U[1] = rho * vx;
-    U[2] = rho * vy;
-    U[3] = rho * vz;
-    U[4] = W[4];
-    U[5] = W[5];
-    U[6] = W[6] / (g - 1.0) + 0.5 * rho * (vx * vx + vy * vy + vz * vz) +
-           0.5 * (Bx * Bx + W[4] * W[4] + W[5] * W[5]);
-    U[7] = W[7];
-}
-
-// x-fluxes of the MHD equations and of E v_x (the advection term of the E equation)
-__device__ __forceinline__ void phys_flux(const double* W, double Bx, double g, double* F) {
-    const double rho = W[0], vx = W[1], vy = W[2], vz = W[3], By = W[4], Bz = W[5];
-    const double p = W[6];
-    const double B2 = Bx * Bx + By * By + Bz * Bz;
-    const double pt = p + 0.5 * B2;
-    const double e = p / (g - 1.0) + 0.5 * rho * (vx * vx + vy * vy + vz * vz) + 0.5 * B2;
-    const double Bv = Bx * vx + By * vy + Bz * vz;
-    F[0] = rho * vx;
-    F[1] = rho * vx * vx + pt - Bx * Bx;
-    F[2] = rho * vx * vy - Bx * By;
-    F[3] = rho * vx * vz - Bx * Bz;
-    F[4] = vx * By - Bx * vy;
-    F[5] = vx * Bz - Bx * vz;
-    F[6] = (e + pt) * vx - Bv * Bx;
-    F[7] = W[7] * vx;
-}
-
-// fast magnetosonic speed from the gas sound speed sqrt(gamma p / rho)
-__device__ __forceinline__ double fast_speed(const double* W, double Bx, double g) {
-    const double rho = W[0];
-    const double cs2 = g * W[6] / rho;
-    const double va2 = (Bx * Bx + W[4] * W[4] + W[5] * W[5]) / rho;
-    const double vax2 = Bx * Bx / rho;
-    const double s = cs2 + va2;
-    return sqrt(0.5 * (s + sqrt(fmax(s * s - 4.0 * cs2 * vax2, 0.0))));
-}
-
 // WENO3 states on both sides of the face between q0 and qp: two two-cell stencils per
 // side with linear weights 1/3 and 2/3 and Jiang-Shu nonlinear weights; the smoothness
-// indicators are divided by the largest square of the four cells (unit-free).
+// indicators are divided by the largest square of the four cells (unit-free). The weights
+// (1/3)/b0^2 and (2/3)/b1^2 are multiplied through by 3 b0^2 b1^2: three divisions in all.
 __device__ __forceinline__ void weno3(double qm, double q0, double qp, double qpp, double& qL,
                                       double& qR) {
     const double eps = 1e-6;
-    const double scale = fmax(fmax(qm * qm, q0 * q0), fmax(qp * qp, qpp * qpp)) + 1e-300;
+    const double is = 1.0 / (fmax(fmax(qm * qm, q0 * q0), fmax(qp * qp, qpp * qpp)) + 1e-300);
     const double dm = q0 - qm, dc = qp - q0, dp = qpp - qp;
-    const double bm = eps + dm * dm / scale, bc = eps + dc * dc / scale, bp = eps + dp * dp / scale;
-    const double a0 = (1.0 / 3.0) / (bm * bm), a1 = (2.0 / 3.0) / (bc * bc);
-    qL = (a0 * (1.5 * q0 - 0.5 * qm) + a1 * (0.5 * q0 + 0.5 * qp)) / (a0 + a1);
-    const double b0 = (1.0 / 3.0) / (bp * bp), b1 = (2.0 / 3.0) / (bc * bc);
-    qR = (b0 * (1.5 * qp - 0.5 * qpp) + b1 * (0.5 * q0 + 0.5 * qp)) / (b0 + b1);
-}
-
-// driving wave at cell centre x and time t, primitive variables
-__device__ __forceinline__ void drive_prim(const Wave1dDev& P, double x, double t, double* W) {
-    const double s = sin(P.k * x - P.omega * t);
-#pragma unroll
-    for (int v = 0; v < 8; ++v) W[v] = P.W0[v] + P.hat[v] * s;
+    const double bm = fma(dm * is, dm, eps), bc = fma(dc * is, dc, eps),
+                 bp = fma(dp * is, dp, eps);
+    const double wm = 2.0 * (bm * bm), wc = bc * bc, wp = 2.0 * (bp * bp);
+    const double mid = fma(0.5, q0, 0.5 * qp);
+    qL = fma(wc, fma(1.5, q0, -0.5 * qm), wm * mid) / (wc + wm);
+    qR = fma(wc, fma(1.5, qp, -0.5 * qpp), wp * mid) / (wc + wp);
 }
 
 // primitive state of cell c: the driving wave left of the grid, zero gradient right of it
@@ -106,124 +45,152 @@ __device__ __forceinline__ void cell_prim(const Wave1dDev& P, const double* __re
 }
 
 __global__ void k_w1_prim(Wave1dDev P, const double* __restrict__ U, double* __restrict__ rho,
-                          double* __restrict__ vx, double* __restrict__ T,
-                          double* __restrict__ T0, double* __restrict__ E) {
+                          double* __restrict__ T, double* __restrict__ T0,
+                          double* __restrict__ E) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P.n) return;
     double W[8];
     cell_prim(P, U, i, 0.0, W);
     const double Tg = W[6] / (W[0] * P.R_gas);
     rho[i] = W[0];
-    vx[i] = W[1];
-    T[i] = Tg;
-    if (T0) T0[i] = Tg;
+    T[i] = T0[i] = Tg;
     E[i] = W[7];
 }
 
-// one thread per face j = 0 .. n (between cells j-1 and j)
-__global__ void k_w1_iface(Wave1dDev P, const double* __restrict__ U, double t,
-                           double* __restrict__ Fi) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j > P.n) return;
-    double Wm[8], W0[8], Wp[8], Wpp[8];
-    cell_prim(P, U, j - 2, t, Wm);
-    cell_prim(P, U, j - 1, t, W0);
-    cell_prim(P, U, j, t, Wp);
-    cell_prim(P, U, j + 1, t, Wpp);
-    double WL[8], WR[8];
-#pragma unroll
-    for (int v = 0; v < 8; ++v) weno3(Wm[v], W0[v], Wp[v], Wpp[v], WL[v], WR[v]);
-    double UL[8], UR[8], FL[8], FR[8];
-    to_cons(WL, P.Bx, P.gamma, UL);
-    to_cons(WR, P.Bx, P.gamma, UR);
-    phys_flux(WL, P.Bx, P.gamma, FL);
-    phys_flux(WR, P.Bx, P.gamma, FR);
-    const double cL = fast_speed(WL, P.Bx, P.gamma), cR = fast_speed(WR, P.Bx, P.gamma);
-    const double SL = fmin(fmin(WL[1] - cL, WR[1] - cR), 0.0);
-    const double SR = fmax(fmax(WL[1] + cL, WR[1] + cR), 0.0);
-    const long long m = P.n + 1;
-#pragma unroll
-    for (int v = 0; v < 8; ++v)
-        Fi[v * m + j] = (SR * FL[v] - SL * FR[v] + SL * SR * (UR[v] - UL[v])) / (SR - SL);
-}
+// A whole explicit evaluation and the state formed from it, one launch in place of five
+// (primitive variables, coupling terms, faces, right-hand side, combination). A line of a few
+// thousand cells is bound by how few threads share its FP64 work, not by memory: one thread a
+// face (7 blocks for 1600 cells) took 101 us for the faces alone. Here a block of four warps
+// owns ADV_C cells and spreads the reconstruction over eight lanes a face, one a variable; 1600
+// cells are 107 blocks. The values pass between the phases through shared memory.
+constexpr int ADV_C = 15, ADV_F = ADV_C + 1, ADV_T = 8 * ADV_F, ADV_P = ADV_C + 4;
 
-// Uout = a U0 + b (Uin + dt L(Uin)), L = -dF/dx + (0, f_r, 0, 0, 0, 0, v.f_r, -P:grad v);
-// the driven cells then take the driving wave at t_stage. Uout may alias U0.
-__global__ void k_w1_stage(Wave1dDev P, const double* U0, const double* __restrict__ Uin,
-                           double* Uout, const double* __restrict__ Fi,
-                           const double* __restrict__ fr, const double* __restrict__ vfr,
-                           const double* __restrict__ pt, double a, double b, double dt,
-                           double t_stage) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P.n) return;
-    const long long n = P.n, m = P.n + 1;
-    if (i < P.nd) {
-        double W[8], u[8];
-        drive_prim(P, (i + 0.5) * P.dx, t_stage, W);
-        to_cons(W, P.Bx, P.gamma, u);
-#pragma unroll
-        for (int v = 0; v < 8; ++v) Uout[v * n + i] = u[v];
-        return;
-    }
-#pragma unroll
-    for (int v = 0; v < 8; ++v) {
-        double dU = -(Fi[v * m + i + 1] - Fi[v * m + i]) / P.dx;
-        if (v == 1) dU += fr[i];
-        if (v == 6) dU += vfr[i];
-        if (v == 7) dU -= pt[i];
-        Uout[v * n + i] = a * U0[v * n + i] + b * (Uin[v * n + i] + dt * dU);
-    }
-}
-
-// L(Uin) = -dF/dx + (0, f_r, 0, 0, 0, 0, v.f_r, -P:grad v), every cell (the driven ones are
-// reset by whatever combines it)
-__global__ void k_w1_rhs(Wave1dDev P, const double* __restrict__ Fi, const double* __restrict__ fr,
-                         const double* __restrict__ vfr, const double* __restrict__ pt,
-                         double* __restrict__ Lout) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P.n) return;
-    const long long n = P.n, m = P.n + 1;
-#pragma unroll
-    for (int v = 0; v < 8; ++v) {
-        double dU = -(Fi[v * m + i + 1] - Fi[v * m + i]) / P.dx;
-        if (v == 1) dU += fr[i];
-        if (v == 6) dU += vfr[i];
-        if (v == 7) dU -= pt[i];
-        Lout[v * n + i] = dU;
-    }
-}
-
-// Uout = U0 + dt (c1 L1 + c2 L2 + c3 L3) + dt (d2 G2 + d3 G3), the G's ([2][n]: gas energy,
-// E) entering variables 6 and 7; null operands have zero weight. Driven cells take the
-// driving wave at t_stage. Uout may alias U0.
-__global__ void k_w1_comb(Wave1dDev P, const double* U0, const double* __restrict__ L1,
-                          const double* __restrict__ L2, const double* __restrict__ L3,
-                          double c1, double c2, double c3, const double* __restrict__ G2,
-                          const double* __restrict__ G3, double d2, double d3, double dt,
-                          double* Uout, double t_stage) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P.n) return;
+__global__ void __launch_bounds__(ADV_T)
+k_w1_advance(Wave1dDev P, W1Stage g) {
+    __shared__ double W[8][ADV_P];             // primitive variables of cells c0-2 .. c0+16
+    __shared__ double Tg[ADV_P];
+    __shared__ double Q[2][8][ADV_F];          // left and right states of the faces
+    __shared__ double Uf[2][8][ADV_F], Ff[2][8][ADV_F], Sp[2][2][ADV_F];
+    __shared__ double Fi[8][ADV_F];
+    __shared__ double src[3][ADV_C];
+    if (g.gate && *g.gate) return;
+    const int c0 = blockIdx.x * ADV_C, tid = threadIdx.x;
     const long long n = P.n;
-    if (i < P.nd) {
-        double W[8], u[8];
-        drive_prim(P, (i + 0.5) * P.dx, t_stage, W);
-        to_cons(W, P.Bx, P.gamma, u);
+    if (tid < ADV_P) {
+        double w[8];
+        cell_prim(P, g.Uin, c0 - 2 + tid, g.t_in, w);
 #pragma unroll
-        for (int v = 0; v < 8; ++v) Uout[v * n + i] = u[v];
-        return;
+        for (int v = 0; v < 8; ++v) W[v][tid] = w[v];
+        Tg[tid] = w[6] / (w[0] * P.R_gas);
     }
+    __syncthreads();
+    {
+        const int f = tid >> 3, v = tid & 7;   // face f lies between cells c0+f-1 and c0+f
+        double l, r;
+        weno3(W[v][f], W[v][f + 1], W[v][f + 2], W[v][f + 3], l, r);
+        Q[0][v][f] = l;
+        Q[1][v][f] = r;
+    }
+    __syncthreads();
+    if (tid < 2 * ADV_F) {
+        // one side of a face: its conserved state, flux and signal speeds
+        const int f = tid % ADV_F, sd = tid / ADV_F;
+        double w[8], u[8], fl[8];
 #pragma unroll
-    for (int v = 0; v < 8; ++v) {
-        double inc = 0.0;
-        if (L1) inc += c1 * L1[v * n + i];
-        if (L2) inc += c2 * L2[v * n + i];
-        if (L3) inc += c3 * L3[v * n + i];
-        if (v >= 6) {
-            if (G2) inc += d2 * G2[(v - 6) * n + i];
-            if (G3) inc += d3 * G3[(v - 6) * n + i];
+        for (int v = 0; v < 8; ++v) w[v] = Q[sd][v][f];
+        to_cons(w, P.Bx, P.gamma, u);
+        phys_flux(w, P.Bx, P.gamma, fl);
+        const double cf = fast_speed(w, P.Bx, P.gamma);
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            Uf[sd][v][f] = u[v];
+            Ff[sd][v][f] = fl[v];
         }
-        Uout[v * n + i] = U0[v * n + i] + dt * inc;
+        Sp[sd][0][f] = w[1] - cf;
+        Sp[sd][1][f] = w[1] + cf;
+    } else if (tid >= 64 && tid < 64 + ADV_C && c0 + tid - 64 < P.n) {
+        // coupling terms of one cell (those of k_coupling on one axis): E's gradient with an
+        // even mirror on the left and a Dirichlet face on the right, the velocity's with
+        // even mirrors on both sides
+        const int q = tid - 64, i = c0 + q;
+        double fr = 0.0, vfr = 0.0, pt = 0.0;
+        if (g.rad) {
+            auto E = [&](int o) {
+                const int c = i + o;
+                if (c < 0) return W[7][-c - 1 - c0 + 2];
+                if (c >= P.n) return 2.0 * g.E_right - W[7][2 * P.n - 1 - c - c0 + 2];
+                return W[7][q + o + 2];
+            };
+            auto vx = [&](int o) {
+                const int c = i + o;
+                return W[1][(c < 0 ? -c - 1 : c >= P.n ? 2 * P.n - 1 - c : c) - c0 + 2];
+            };
+            const double ih = 1.0 / (12.0 * P.dx);
+            const double Ec = E(0), r = W[0][q + 2];
+            const double t = g.op.kind == FLD_OPACITY_CONST ? 1.0 : Tg[q + 2];
+            bool ok = pos_finite(Ec) && pos_finite(r) && pos_finite(t);
+            const double kap = ok ? opacity_eval(g.op, r, t) : 0.0;
+            ok = ok && pos_finite(kap);
+            if (ok) {
+                const double gr = ((E(-2) - 8.0 * E(-1)) + 8.0 * E(1) - E(2)) * ih;
+                const double dv = ((vx(-2) - 8.0 * vx(-1)) + 8.0 * vx(1) - vx(2)) * ih;
+                const double R = sqrt(gr * gr) / (kap * r * Ec);
+                const double lam = g.mode == FLD_LIMITER_LP
+                                       ? (2.0 + R) / (6.0 + 3.0 * R + R * R)
+                                       : g.mode == FLD_LIMITER_MINERBO ? minerbo_lambda(R)
+                                                                       : 1.0 / 3.0;
+                const double f = lam + lam * lam * R * R;
+                fr = -lam * gr;
+                vfr = vx(0) * fr;
+                // P_xx = E f where the gradient has a direction, E (1 - f)/2 where it vanishes
+                pt = (gr != 0.0 ? f : 0.5 * (1.0 - f)) * Ec * dv;
+            } else {
+                atomicOr(g.err, ERRBIT_DOMAIN);
+            }
+        }
+        src[0][q] = fr;
+        src[1][q] = vfr;
+        src[2][q] = pt;
     }
+    __syncthreads();
+    {
+        const int f = tid >> 3, v = tid & 7;
+        const double SL = fmin(fmin(Sp[0][0][f], Sp[1][0][f]), 0.0);
+        const double SR = fmax(fmax(Sp[0][1][f], Sp[1][1][f]), 0.0);
+        Fi[v][f] = (SR * Ff[0][v][f] - SL * Ff[1][v][f] +
+                    SL * SR * (Uf[1][v][f] - Uf[0][v][f])) / (SR - SL);
+    }
+    __syncthreads();
+    const int v = tid / ADV_F, q = tid % ADV_F, i = c0 + q;    // consecutive cells a half-warp
+    if (q >= ADV_C || i >= P.n) return;
+    const long long at = v * n + i;
+    double dU = -(Fi[v][q + 1] - Fi[v][q]) / P.dx;
+    if (v == 1) dU += src[0][q];
+    if (v == 6) dU += src[1][q];
+    if (v == 7) dU -= src[2][q];
+    if (g.Lout) g.Lout[at] = dU;
+    double out;
+    if (i < P.nd) {
+        double w[8], u[8];
+        drive_prim(P, (i + 0.5) * P.dx, g.t_out, w);
+        to_cons(w, P.Bx, P.gamma, u);
+        out = u[0];
+#pragma unroll
+        for (int e = 1; e < 8; ++e) out = v == e ? u[e] : out;
+    } else if (g.ssp) {
+        out = g.a * g.U0[at] + g.b * (g.Uin[at] + g.dt * dU);
+    } else {
+        double inc = 0.0;
+        if (g.La) inc += g.ca * g.La[at];
+        if (g.Lb) inc += g.cb * g.Lb[at];
+        inc += g.cn * dU;
+        if (v >= 6) {
+            if (g.G2) inc += g.d2 * g.G2[(v - 6) * n + i];
+            if (g.G3) inc += g.d3 * g.G3[(v - 6) * n + i];
+        }
+        out = g.U0[at] + g.dt * inc;
+    }
+    g.Uout[at] = out;
 }
 
 // the implicit increment of a stage: G = (Uafter - Ubefore) / tau for variables 6, 7
@@ -283,38 +250,18 @@ int blocks_for(long long n) { return (int)((n + W1_THREADS - 1) / W1_THREADS); }
 
 }  // namespace
 
-void launch_w1_prim(const Wave1dDev& P, const double* U, double* rho, double* vx, double* T,
-                    double* T0, double* E, cudaStream_t s) {
-    k_w1_prim<<<blocks_for(P.n), W1_THREADS, 0, s>>>(P, U, rho, vx, T, T0, E);
+void launch_w1_prim(const Wave1dDev& P, const double* U, double* rho, double* T, double* T0,
+                    double* E, cudaStream_t s) {
+    k_w1_prim<<<blocks_for(P.n), W1_THREADS, 0, s>>>(P, U, rho, T, T0, E);
 }
 
-void launch_w1_iface(const Wave1dDev& P, const double* U, double t, double* Fi, cudaStream_t s) {
-    k_w1_iface<<<blocks_for(P.n + 1), W1_THREADS, 0, s>>>(P, U, t, Fi);
-}
-
-void launch_w1_stage(const Wave1dDev& P, const double* U0, const double* Uin, double* Uout,
-                     const double* Fi, const double* fr, const double* vfr, const double* pt,
-                     double a, double b, double dt, double t_stage, cudaStream_t s) {
-    k_w1_stage<<<blocks_for(P.n), W1_THREADS, 0, s>>>(P, U0, Uin, Uout, Fi, fr, vfr, pt, a, b,
-                                                       dt, t_stage);
+void launch_w1_advance(const Wave1dDev& P, const W1Stage& g, cudaStream_t s) {
+    k_w1_advance<<<(P.n + ADV_C - 1) / ADV_C, ADV_T, 0, s>>>(P, g);
 }
 
 void launch_w1_post(const Wave1dDev& P, double* U, const double* rho, const double* T0,
                     const double* T, const double* E, double t, cudaStream_t s) {
     k_w1_post<<<blocks_for(P.n), W1_THREADS, 0, s>>>(P, U, rho, T0, T, E, t);
-}
-
-void launch_w1_rhs(const Wave1dDev& P, const double* Fi, const double* fr, const double* vfr,
-                   const double* pt, double* Lout, cudaStream_t s) {
-    k_w1_rhs<<<blocks_for(P.n), W1_THREADS, 0, s>>>(P, Fi, fr, vfr, pt, Lout);
-}
-
-void launch_w1_comb(const Wave1dDev& P, const double* U0, const double* L1, const double* L2,
-                    const double* L3, double c1, double c2, double c3, const double* G2,
-                    const double* G3, double d2, double d3, double dt, double* Uout,
-                    double t_stage, cudaStream_t s) {
-    k_w1_comb<<<blocks_for(P.n), W1_THREADS, 0, s>>>(P, U0, L1, L2, L3, c1, c2, c3, G2, G3, d2,
-                                                      d3, dt, Uout, t_stage);
 }
 
 void launch_w1_incr(const Wave1dDev& P, const double* Ua, const double* Ub, double inv_tau,
