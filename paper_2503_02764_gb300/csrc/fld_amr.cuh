@@ -22,14 +22,29 @@ struct AmrGeom {
 void launch_amr_setup(const AmrGeom& G, const double* Dc, const double* Df, const double* Ec,
                       const double* Ef, const double* Ebc, double* bc, double* bf, double* DH,
                       cudaStream_t s);
-void launch_amr_smooth(const AmrGeom& G, int phase, const double* Dc, const double* Df,
+// Rows of one grid, formed once per solve: face conductances per axis (extent + 1 along it)
+// and inverse diagonals.
+struct AmrRows {
+    double* w[3];
+    double* inv;
+};
+// x: readable values of both grids (their faces are walked, the values not used)
+void launch_amr_rows(const AmrGeom& G, const AmrRows& Rc, const AmrRows& Rf, const double* Dc,
+                     const double* Df, const double* xc, const double* xf, cudaStream_t s);
+void launch_amr_smooth(const AmrGeom& G, const AmrRows& Rc, const AmrRows& Rf, int phase,
                        const double* bc, const double* bf, double* xc, double* xf,
                        cudaStream_t s);
-int launch_amr_resid(const AmrGeom& G, const double* Dc, const double* Df, const double* bc,
+int launch_amr_resid(const AmrGeom& G, const AmrRows& Rc, const AmrRows& Rf, const double* bc,
                      const double* bf, const double* xc, const double* xf, double* rc, double* rf,
                      double* partials, int nblocks, cudaStream_t s);
 void launch_amr_average(const AmrGeom& G, const double* vf, double* vc, cudaStream_t s);
 void launch_amr_correct(const AmrGeom& G, const double* e, double* xc, double* xf,
                         cudaStream_t s);
+
+// The block's multigrid as the coarse correction (fld_api.cu): the operator of D over dt set up
+// once per solve, then `cycles` V-cycles on A e = r from e = 0, without a read-back.
+fld_status fld_correction_setup(fld_handle* h, double dt, const double* D, const double* r,
+                                cudaStream_t s);
+fld_status fld_correction(fld_handle* h, const double* r, double* e, int cycles, cudaStream_t s);
 
 }  // namespace fld

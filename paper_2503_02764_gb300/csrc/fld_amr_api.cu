@@ -20,6 +20,7 @@ struct fld_amr {
     long long nC = 0, nF = 0;
     int nblk = 0;
     double *bc = nullptr, *bf = nullptr, *rc = nullptr, *rf = nullptr;
+    AmrRows Rc = {}, Rf = {};
     double *eH = nullptr, *DH = nullptr, *zero_faces = nullptr, *partials = nullptr;
     double *sum = nullptr, *hsum = nullptr;   // device scalar, pinned host copy
     std::vector<void*> allocs;
@@ -28,7 +29,13 @@ struct fld_amr {
 namespace {
 
 constexpr int AMR_SWEEPS = 2;          // composite red-black sweeps after each correction
-constexpr double AMR_COARSE_TOL = 1e-6;
+// The coarse correction is a fixed number of V-cycles: the composite iteration contracts by
+// about 0.1 a cycle whether the block is solved to 1e-6 (four to five V-cycles and as many
+// read-backs, what it took before) or by one V-cycle. Where a cycle contracts by less than
+// AMR_SLOW, the block's V-cycles are what limits it, and their number doubles up to AMR_MOST.
+constexpr int AMR_CYCLES = 1, AMR_MOST = 16;
+constexpr double AMR_SLOW = 0.25;
+constexpr double AMR_COARSE_TOL = 1e-6;   // 1D blocks: the direct solve's tolerance
 
 bool dal(fld_amr* a, double** q, long long n) {
     void* m = nullptr;
@@ -143,7 +150,10 @@ fld_status fld_amr_create(fld_amr** out, const fld_grid* g, const fld_patch* pat
     bool ok = dal(a, &a->bc, nC) && dal(a, &a->bf, nF) && dal(a, &a->rc, nC) &&
               dal(a, &a->rf, nF) && dal(a, &a->eH, nC) && dal(a, &a->DH, nC) &&
               dal(a, &a->zero_faces, nfaces) && dal(a, &a->partials, a->nblk) &&
-              dal(a, &a->sum, 1);
+              dal(a, &a->sum, 1) && dal(a, &a->Rc.inv, nC) && dal(a, &a->Rf.inv, nF);
+    for (int d = 0; d < g->ndim; ++d)
+        ok = ok && dal(a, &a->Rc.w[d], nC / G.nc[d] * (G.nc[d] + 1)) &&
+             dal(a, &a->Rf.w[d], nF / G.nf[d] * (G.nf[d] + 1));
     if (ok && cudaMallocHost(&a->hsum, sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         a->hsum = nullptr;
@@ -182,45 +192,55 @@ fld_status fld_amr_diffuse(fld_amr* a, double dt, const double* Dc, const double
     AmrGeom& G = a->G;
     G.dt = dt;
     launch_amr_setup(G, Dc, Df, Ec, Ef, E_bc, a->bc, a->bf, a->DH, s);
-    launch_sumsq(a->nC, a->bc, a->partials, a->nblk, s);
+    launch_sumsq(a->nC, a->bc, a->partials, a->nblk / 2, s);
     note_launches(2);
-    double b2c = 0.0, b2f = 0.0;
-    fld_status rc = reduce(a, a->nblk, s, &b2c);
+    launch_sumsq(a->nF, a->bf, a->partials + a->nblk / 2, a->nblk / 2, s);
+    launch_amr_rows(G, a->Rc, a->Rf, Dc, Df, Ec, Ef, s);
+    note_launches(5);
+    double b2 = 0.0;
+    fld_status rc = reduce(a, a->nblk / 2 * 2, s, &b2);
     if (rc) return rc;
-    launch_sumsq(a->nF, a->bf, a->partials, a->nblk, s);
-    note_launches(1);
-    rc = reduce(a, a->nblk, s, &b2f);
-    if (rc) return rc;
-    const double bnorm = std::sqrt(b2c + b2f);
+    const double bnorm = std::sqrt(b2);
     if (st) {
         memset(st, 0, sizeof(*st));
         st->levels = fld_num_levels(a->hc) + 1;
     }
     int cyc = 0;
+    int vcycles = AMR_CYCLES;
     double rel = 0.0;
     for (;;) {
-        const int nb = launch_amr_resid(G, Dc, Df, a->bc, a->bf, Ec, Ef, a->rc, a->rf,
+        const int nb = launch_amr_resid(G, a->Rc, a->Rf, a->bc, a->bf, Ec, Ef, a->rc, a->rf,
                                         a->partials, a->nblk, s);
-        note_launches(1);
+        note_launches(2);
         double r2;
         rc = reduce(a, nb, s, &r2);
         if (rc) return rc;
+        const double before = rel;
         rel = bnorm > 0 ? std::sqrt(r2) / bnorm : 0.0;
         if (st && cyc < 64) st->resid_hist[cyc] = rel;
         if (!(rel > a->o.tol) || cyc >= a->o.max_cycles || !std::isfinite(rel)) break;
         // coarse correction: the restricted residual on the whole block, solved by the
         // block's multigrid (homogeneous walls), added on the composite grid
         launch_amr_average(G, a->rf, a->rc, s);
-        rc = ck(cudaMemcpyAsync(a->eH, a->rc, sizeof(double) * a->nC, cudaMemcpyDeviceToDevice,
-                                s));
-        if (rc) return rc;
         note_launches(1);
-        const fld_status cs = fld_diffuse(a->hc, dt, a->DH, a->zero_faces, a->eH, nullptr, stream);
-        if (cs != FLD_OK && cs != FLD_ERR_NOT_CONVERGED) return cs;
+        if (a->g.ndim == 1) {
+            rc = ck(cudaMemcpyAsync(a->eH, a->rc, sizeof(double) * a->nC,
+                                    cudaMemcpyDeviceToDevice, s));
+            if (rc) return rc;
+            const fld_status cs = fld_diffuse(a->hc, dt, a->DH, a->zero_faces, a->eH, nullptr,
+                                              stream);
+            if (cs != FLD_OK && cs != FLD_ERR_NOT_CONVERGED) return cs;
+        } else {
+            if (cyc == 0) rc = fld_correction_setup(a->hc, dt, a->DH, a->rc, s);
+            else if (rel > AMR_SLOW * before) vcycles = std::min(2 * vcycles, AMR_MOST);
+            if (rc == FLD_OK) rc = fld_correction(a->hc, a->rc, a->eH, vcycles, s);
+            if (rc != FLD_OK) return rc;
+        }
         launch_amr_correct(G, a->eH, Ec, Ef, s);
         note_launches(1);
         for (int i = 0; i < AMR_SWEEPS; ++i)
-            for (int ph = 0; ph < 4; ++ph) launch_amr_smooth(G, ph, Dc, Df, a->bc, a->bf, Ec, Ef, s);
+            for (int ph = 0; ph < 4; ++ph)
+                launch_amr_smooth(G, a->Rc, a->Rf, ph, a->bc, a->bf, Ec, Ef, s);
         note_launches(4 * AMR_SWEEPS);
         ++cyc;
     }

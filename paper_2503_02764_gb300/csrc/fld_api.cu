@@ -11,6 +11,7 @@
 #include <new>
 #include <vector>
 
+#include "fld_amr.cuh"
 #include "fld_internal.cuh"
 #include "fld_line.cuh"
 #include "fld_wave1d.cuh"
@@ -581,6 +582,16 @@ void restrict_pyramid(fld_handle* h, LevelBufs<T>* P, cudaStream_t s) {
         });
 }
 
+// the coarser levels' K, and the FP64 V-cycle's coefficients
+void setup_pyramid(fld_handle* h, bool mixed, cudaStream_t s) {
+    if (mixed) return restrict_pyramid<float>(h, h->d32, s);
+    restrict_pyramid<double>(h, h->d64, s);
+    for (int l = 0; l < h->nlev; ++l)
+        if (h->w64[l].inv)
+            run(h, "coef64", l, h->lv[l].ncell, s,
+                [&] { launch_coef64(h->lv[l], h->d64[l].K, h->w64[l], s); });
+}
+
 fld_status read_scalars(fld_handle* h, cudaStream_t s, double* sum, unsigned* err) {
     FLD_CK(cudaMemcpyAsync(h->hscal, h->scal, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
     FLD_CK(cudaStreamSynchronize(s));
@@ -870,16 +881,7 @@ fld_status diffuse_impl(fld_handle* h, double dt, const double* D, const double*
                            mixed ? h->d32[0].K : nullptr, h->d64[0].b, &h->scal->err,
                            want_kmax ? &h->scal->kmax : nullptr, s);
     });
-    if (!direct) {
-        if (mixed) restrict_pyramid<float>(h, h->d32, s);
-        else {
-            restrict_pyramid<double>(h, h->d64, s);
-            for (int l = 0; l < h->nlev; ++l)
-                if (h->w64[l].inv)
-                    run(h, "coef64", l, h->lv[l].ncell, s,
-                        [&] { launch_coef64(h->lv[l], h->d64[l].K, h->w64[l], s); });
-        }
-    }
+    if (!direct) setup_pyramid(h, mixed, s);
     run(h, "sumsq", 0, L0.ncell, s,
         [&] { launch_sumsq(L0.ncell, h->d64[0].b, h->partials, h->norm_blocks, s); });
     run(h, "finish_sum", 0, h->norm_blocks, s,
@@ -1358,6 +1360,56 @@ fld_status fld_step(fld_handle* h, const fld_consts* k, const fld_opacity* op, d
 }  // extern "C"
 
 long long fld::fld_handle_cells(const fld_handle* h) { return h ? h->ncell : 0; }
+
+// ---- the composite grid's coarse correction (fld_amr_api.cu), 2D and 3D
+fld_status fld::fld_correction_setup(fld_handle* h, double dt, const double* D, const double* r,
+                                     cudaStream_t s) {
+    const Lvl& L0 = h->lv[0];
+    const bool mixed = h->o.precision != FLD_PREC_FP64;
+    const bool want_kmax = h->o.truncate;
+    if (want_kmax) FLD_CK(cudaMemsetAsync(&h->scal->kmax, 0, sizeof(unsigned), s));
+    run(h, "prep", 0, L0.ncell, s, [&] {
+        launch_prep_level0(L0, dt / (h->g.h[0] * h->g.h[0]), D, r, nullptr, h->bc_off,
+                           h->d64[0].K, mixed ? h->d32[0].K : nullptr, h->d64[0].b,
+                           &h->scal->err, want_kmax ? &h->scal->kmax : nullptr, s);
+    });
+    setup_pyramid(h, mixed, s);
+    FLD_CK(cudaGetLastError());
+    double sum;
+    unsigned err;
+    const fld_status rc = read_scalars(h, s, &sum, &err);
+    if (rc != FLD_OK) return rc;
+    if (err) {
+        cudaMemsetAsync(&h->scal->err, 0, sizeof(unsigned), s);
+        return FLD_ERR_DOMAIN;
+    }
+    float kf;
+    memcpy(&kf, &h->hscal->kmax, sizeof(kf));
+    choose_depth(h, want_kmax ? (double)kf : -1.0);
+    return FLD_OK;
+}
+
+fld_status fld::fld_correction(fld_handle* h, const double* r, double* e, int cycles,
+                               cudaStream_t s) {
+    const long long n = h->ncell;
+    if (h->o.precision == FLD_PREC_FP64) {
+        FLD_CK(cudaMemcpyAsync(h->d64[0].b, r, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+        FLD_CK(cudaMemsetAsync(e, 0, sizeof(double) * n, s));
+        h->d64[0].x = e;
+        for (int c = 0; c < cycles; ++c) vcycle<double>(h, h->d64, 0, s);
+    } else {
+        run(h, "to_f32", 0, n, s, [&] { launch_to_f32(n, r, h->d32[0].b, s); });
+        const int inner = h->o.inner;
+        h->o.inner = cycles;
+        const fld_status rc = vcycle32(h, s);
+        h->o.inner = inner;
+        if (rc != FLD_OK) return rc;
+        FLD_CK(cudaMemsetAsync(e, 0, sizeof(double) * n, s));
+        run(h, "add_correction", 0, n, s, [&] { launch_add_correction(n, e, h->d32[0].x, s); });
+    }
+    FLD_CK(cudaGetLastError());
+    return FLD_OK;
+}
 
 // ---- the wave step's implicit stage (fld_wave1d_api.cu)
 bool fld::fld_line_wave_ok(const fld_handle* h) { return line_step_ok(h) && !h->o.diag; }

@@ -492,6 +492,16 @@ void launch_add_correction(long long n, double* x, const float* e, cudaStream_t 
     k_add_correction<<<grid_for(n, 256), 256, 0, s>>>(n, x, e);
 }
 
+__global__ void k_to_f32(long long n, const double* __restrict__ v, float* __restrict__ f) {
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
+         p += (long long)gridDim.x * blockDim.x)
+        f[p] = (float)v[p];
+}
+
+void launch_to_f32(long long n, const double* v, float* f, cudaStream_t s) {
+    k_to_f32<<<grid_for(n, 256), 256, 0, s>>>(n, v, f);
+}
+
 __global__ void k_sumsq(long long n, const double* __restrict__ v, double* __restrict__ partials) {
     __shared__ double sh[32];
     double a = 0.0;
