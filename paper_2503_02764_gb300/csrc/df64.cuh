@@ -137,6 +137,15 @@ __device__ __forceinline__ double df_to_double(df x) { return (double)x.hi + (do
 // the double's significand rounded to 24 bits (ties to even, a carry moving it to the next
 // binade); the remainder v - hi is an integer number of the double's ulps below 2^29,
 // rounded to 24 bits by the int -> float conversion and scaled through its exponent field.
+//
+// f32_of_int: the FP32 number nearest to a 32-bit integer, ties to even, from two
+// exact pieces and one FMA: the conversion instruction holds the FP64 pipe of this GPU for as
+// long as two FP64 instructions.
+__device__ __forceinline__ float f32_of_int(int v) {
+    const float hi = __uint_as_float(0x4B400000u + (unsigned)(v >> 14)) - 12582912.f;
+    const float lo = __uint_as_float(0x4B400000u + (unsigned)(v & 0x3FFF)) - 12582912.f;
+    return __fmaf_rn(hi, 16384.f, lo);
+}
 __device__ __forceinline__ bool df_split_i(double v, int k2, df& out) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     const unsigned sgn = (unsigned)(b >> 63);
@@ -160,7 +169,7 @@ __device__ __forceinline__ bool df_split_i(double v, int k2, df& out) {
         out.lo = 0.f;
         return true;
     }
-    unsigned fb = __float_as_uint(__int2float_rn((int)du));
+    unsigned fb = __float_as_uint(f32_of_int((int)du));
     fb = (fb & 0x807FFFFFu) | ((unsigned)((int)((fb >> 23) & 0xFF) + (e - 1075)) << 23);
     const float lo = __uint_as_float(fb);
     out.lo = sgn ? -lo : lo;

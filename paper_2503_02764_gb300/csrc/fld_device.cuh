@@ -3,6 +3,7 @@
 // block reductions, limiter ghost values and the exchange root.
 #pragma once
 #include "df64.cuh"
+#include "fix64.cuh"
 #include "fld_internal.cuh"
 
 namespace fld {
@@ -170,6 +171,26 @@ __device__ __forceinline__ double fetch_E(const Lvl& L, const double* __restrict
     return v;
 }
 
+// The four values E_-2, E_-1, E_+1, E_+2 along axis d: straight from memory two cells or more
+// from the axis's ends, through the ghost rules elsewhere.
+__device__ __forceinline__ void fetch_axis(const Lvl& L, const double* __restrict__ E,
+                                           const double* __restrict__ Ebc, const BcOff& bo, int i,
+                                           int j, int k, int d, int p, double v[4]) {
+    const int c = d == 0 ? i : d == 1 ? j : k;
+    if (c >= 2 && c < L.n[d] - 2) {
+        const int st = d == 0 ? 1 : d == 1 ? L.n[0] : L.n[0] * L.n[1];
+        v[0] = E[fld_at(p - 2 * st, L.ncell)];
+        v[1] = E[fld_at(p - st, L.ncell)];
+        v[2] = E[fld_at(p + st, L.ncell)];
+        v[3] = E[fld_at(p + 2 * st, L.ncell)];
+    } else {
+        v[0] = fetch_E(L, E, Ebc, bo, i, j, k, d, -2);
+        v[1] = fetch_E(L, E, Ebc, bo, i, j, k, d, -1);
+        v[2] = fetch_E(L, E, Ebc, bo, i, j, k, d, 1);
+        v[3] = fetch_E(L, E, Ebc, bo, i, j, k, d, 2);
+    }
+}
+
 // Minerbo's limiter (the paper implements it but does not print it; the published closed
 // form): 2 / (3 + sqrt(9 + 12 R^2)) for R <= 3/2, 1 / (1 + R + sqrt(1 + 2R)) above; both
 // branches give 2/9 and the same slope at R = 3/2, and lambda R -> 1 as R -> infinity.
@@ -273,16 +294,75 @@ __device__ __forceinline__ double exchange_root(double alpha, double beta, doubl
     return x;
 }
 
+// kappa rho of a cell with positive finite rho and T; false if kappa is not positive and finite.
+// The Kramers-like law kappa0 rho T^-3.5 as kappa0 rho^2 / (T^3 sqrt(T)): nine FP64
+// instructions (fourteen with T^-1/2 refined in FP64 and raised to its seventh power).
+template <bool kTables>
+__device__ __forceinline__ bool kapparho(const Opacity& op, double r, double t, double& kr) {
+    if (op.kind == FLD_OPACITY_POWER && op.a_rho == 1.0 && op.a_T == -3.5 && in_f32_range(t)) {
+        const double t2 = t * t;
+        const double q = t2 * t * fix_sqrt(t), n = op.kappa0 * r;
+        if (div_ok(n, q)) {
+            const double kap = fix_div(n, q);
+            kr = kap * r;
+            return pos_finite(kap);
+        }
+    }
+    const double kap = opacity_eval<kTables>(op, r, t);
+    kr = kap * r;
+    return pos_finite(kap);
+}
+
 // ----------------------------------------------------------------- limiter, one cell
 // R = |grad E| / (kappa rho E) (Eq. fld_R), lambda = (2 + R)/(6 + 3R + R^2)
 // (Eq. fld_lambda), D = c lambda / (kappa rho) (Eq. fld_F), grad E by the 5-point
 // 4th-order difference. With a = kappa rho E and g = |grad E| (R = g/a), multiplying the
 // limiter's numerator and denominator by a^2 gives
-//   D = c E (2a + g) / (6a^2 + 3ag + g^2),
-// one square root and one division (FP32-seeded Newton-Raphson where the operands allow
-// it): FP64 issues at a small fraction of the FP32 rate here. Minerbo's limiter and
-// operands outside the FP32 range take R itself. kr_out receives kappa rho (the exchange
-// of the same substep reuses it). Returns false on a domain error.
+//   D = c E (2a + g) / (3a (2a + g) + g^2),
+// and Minerbo's likewise c E 2 / (3a + sqrt(9a^2 + 12 g^2)) for g <= 3a/2, else
+// c E / (a + g + sqrt(a^2 + 2 a g)): one or two square roots and one division, by the routines
+// of fix64.cuh where the operands allow it (FP64 issues at a small fraction of the FP32 rate
+// here: LP with a Kramers opacity took 46 FP64 instructions with the gradient in FP64 and
+// Newton-Raphson roots, and takes 23). Operands outside the FP32 range take R itself. kr_out
+// receives kappa rho (the exchange of the same substep reuses it). Returns false on a domain
+// error.
+//
+// The quotient q = lambda / a (LP or Minerbo) of a = kappa rho E and g2 = |grad E|^2, lambda
+// itself with want_lm (by its own division: a's rounding then cancels), and, with LP or NEED_G, g;
+// false where an operand leaves the FP32 range.
+template <bool NEED_G = false>
+__device__ __forceinline__ bool limiter_core(double a, double g2, int mode, double one,
+                                             bool want_lm, double& g, double& q, double& lm) {
+    const bool gzero = __double_as_longlong(g2) == 0;
+    if (!(in_f32_range(a) && (gzero || in_f32_range(g2)))) return false;
+    double num, den;
+    g = 0.0;
+    if (mode == FLD_LIMITER_LP) {
+        if (!gzero) g = fix_sqrt(g2);
+        num = fma(2.0, a, g);
+        den = fma(3.0 * a, num, g2);
+    } else {
+        // the branch g <= 3a/2 by integer comparison of g^2 with 9/4 a^2 (positive numbers
+        // order as their bits); it is the formula's own up to the rounding of a^2
+        const double aa = a * a;
+        const bool low = gzero ||
+                         __double_as_longlong(g2) <= __double_as_longlong(2.25 * aa);
+        if (!gzero && (NEED_G || !low)) g = fix_sqrt(g2);
+        const double under = low ? fma(9.0, aa, 12.0 * g2) : a * fma(2.0, g, a);
+        const double root = in_f32_range(under) ? fix_sqrt(under) : sqrt(under);
+        den = low ? fma(3.0, a, root) : fma(g, one, a);
+        if (!low) den = fma(root, one, den);
+        num = low ? 2.0 : 1.0;
+    }
+    if (!div_ok(num, den)) return false;
+    q = fix_div(num, den);
+    if (want_lm) {
+        const double an = a * num;
+        lm = div_ok(an, den) ? fix_div(an, den) : an / den;
+    }
+    return true;
+}
+
 template <bool kTables = true>
 __device__ __forceinline__ bool limiter_cell(const Lvl& L, const double* ih,
                                              const double* __restrict__ E,
@@ -295,79 +375,66 @@ __device__ __forceinline__ bool limiter_cell(const Lvl& L, const double* ih,
                                              double one = 1.0) {
     const double Ec = E[p], r = rho[p];
     const double t = (op.kind == FLD_OPACITY_CONST) ? 1.0 : T[p];
-    const double kap = opacity_eval<kTables>(op, r, t);
-    if (!(pos_finite(Ec) && pos_finite(r) && pos_finite(t) && pos_finite(kap))) return false;
-    const double kr = kap * r;
+    double kr;
+    if (!(pos_finite(Ec) && pos_finite(r) && pos_finite(t))) return false;
+    if (!kapparho<kTables>(op, r, t, kr)) return false;
     if (kr_out) *kr_out = kr;
-    double lm = 1.0 / 3.0;
-    if (mode != FLD_LIMITER_DIFFUSION) {
-        double g2 = 0.0;
-        // unrolled over the three axes, so that every index into the level and the
-        // spacings is a constant (no local-memory copy of them)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            if (d >= L.ndim) break;
-            const double em2 = fetch_E(L, E, Ebc, bo, i, j, k, d, -2);
-            const double em1 = fetch_E(L, E, Ebc, bo, i, j, k, d, -1);
-            const double ep1 = fetch_E(L, E, Ebc, bo, i, j, k, d, 1);
-            const double ep2 = fetch_E(L, E, Ebc, bo, i, j, k, d, 2);
-            // (E_-2 - 8 E_-1) + 8 E_+1 - E_+2 as three FMAs (`one` = 1.0 from the kernel's
-            // arguments: an FP64 add costs the FP64 pipe twice an FMA's time on this GPU)
-            const double g = fma(ep2, -one, fma(8.0, ep1, fma(-8.0, em1, em2))) * ih[d];
-            g2 = fma(g, g, g2);
-        }
-        const double a = kr * Ec;
-        const bool gzero = __double_as_longlong(g2) == 0;
-        if (mode == FLD_LIMITER_LP && in_f32_range(a) && (gzero || in_f32_range(g2))) {
-            const double g = gzero ? 0.0 : sqrt_nr(g2);
-            const double den = fma(a, fma(6.0, a, 3.0 * g), g2);
-            const double n2 = fma(2.0, a, g);
-            if (in_f32_range(den)) {
-                Dout = div_nr((c * Ec) * n2, den);
-                if (want_lm) lmout = div_nr(a * n2, den);
-                return true;
-            }
-        }
-        if (in_f32_range(a) && (gzero || in_f32_range(g2))) {
-            const double v = rcp_nr(a);
-            const double R = gzero ? 0.0 : sqrt_nr(g2) * v;
-            if (mode == FLD_LIMITER_MINERBO) {
-                lmout = minerbo_lambda(R);
-            } else {
-                const double P = 2.0 + R, Q = fma(R, R + 3.0, 6.0);
-                const double rQ = in_f32_range(Q) ? rcp_nr(Q) : 1.0 / Q;
-                lmout = P * rQ;
-            }
-            Dout = c * lmout * (Ec * v);
-            return true;
-        }
-        const double R = sqrt(g2) / a;
-        lm = mode == FLD_LIMITER_MINERBO ? minerbo_lambda(R) : (2.0 + R) / (6.0 + 3.0 * R + R * R);
+    if (mode == FLD_LIMITER_DIFFUSION) {
+        lmout = 1.0 / 3.0;
+        const double cl = c * lmout;
+        Dout = div_ok(cl, kr) ? fix_div(cl, kr) : cl / kr;
+        return true;
     }
-    lmout = lm;
-    Dout = in_f32_range(kr) ? c * lm * rcp_nr(kr) : c * lm / kr;
+    double g2 = 0.0;
+    // unrolled over the three axes, so that every index into the level and the spacings is
+    // a constant (no local-memory copy of them)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        if (d >= L.ndim) break;
+        double v[4];
+        fetch_axis(L, E, Ebc, bo, i, j, k, d, (int)p, v);
+        const double g = fix_stencil(v[0], v[1], v[2], v[3]) * ih[d];
+        g2 = fma(g, g, g2);
+    }
+    const double a = kr * Ec;
+    double g, q;
+    if (limiter_core(a, g2, mode, one, want_lm, g, q, lmout)) {
+        Dout = c * Ec * q;
+        return true;
+    }
+    const double R = sqrt(g2) / a;
+    lmout = mode == FLD_LIMITER_MINERBO ? minerbo_lambda(R) : (2.0 + R) / (6.0 + 3.0 * R + R * R);
+    Dout = in_f32_range(kr) ? c * lmout * rcp_nr(kr) : c * lmout / kr;
     return true;
 }
 
 // ----------------------------------------------------------------- exchange, one cell
 // Backward Euler on de/dt = +qdot, dE/dt = -qdot (Eqs. heating, qdot), given
-// kr = kappa rho (frozen at the step's start): chi = dt c kr, solves
-// alpha T' + beta T'^4 = q (exchange_root) with alpha = rho c_v, beta = a_r chi/(1+chi),
-// q = alpha T + chi E/(1+chi), and sets E' = (E + chi a_r T'^4)/(1 + chi)
-// = E/(1+chi) + beta T'^4. The caller checks r, t, er and kr.
+// kr = kappa rho (frozen at the step's start). With chi = dt c kr and everything multiplied by
+// 1 + chi, T' is the root of A T' + B T'^4 = Q with A = rho c_v (1 + chi), B = a_r chi,
+// Q = A T + chi E (exchange_root), and E' = (E + B T'^4) / (1 + chi): one division in all, after
+// the root (17 FP64 instructions; the form with chi/(1 + chi) took 24). The caller checks r,
+// t, er and kr.
 __device__ __forceinline__ void exchange_cell_kr(double r, double kr, double& t, double& er,
                                                  double dtc, double a_r, double cv,
                                                  double one = 1.0) {
     const double chi = dtc * kr;
-    const double alpha = r * cv;
-    const double d1 = fma(chi, one, 1.0);      // 1 + chi as an FMA (see limiter_cell)
-    const double inv1 = in_f32_range(d1) ? rcp_nr(d1) : 1.0 / d1;
-    const double w = chi * inv1;
-    const double beta = w * a_r;
-    const double q = fma(w, er, alpha * t);
-    const double x = exchange_root(alpha, beta, q);
+    const double d1 = fma(chi, one, 1.0);      // 1 + chi as an FMA (an FP64 add costs two)
+    if (!in_f32_range(d1)) {                   // divided by 1 + chi: nothing overflows
+        const double inv1 = 1.0 / d1, w = chi * inv1;
+        const double beta = w * a_r, q = fma(w, er, r * cv * t);
+        const double x = exchange_root(r * cv, beta, q), x2 = x * x;
+        er = fma(beta, x2 * x2, er * inv1);
+        t = x;
+        return;
+    }
+    const double A = r * cv * d1;
+    const double B = a_r * chi;
+    const double Q = fma(chi, er, A * t);
+    const double x = exchange_root(A, B, Q);
     const double x2 = x * x;
-    er = fma(beta, x2 * x2, er * inv1);
+    const double N = fma(B, x2 * x2, er);
+    er = div_ok(N, d1) ? fix_div(N, d1) : N / d1;
     t = x;
 }
 
@@ -377,9 +444,9 @@ template <bool kTables = true>
 __device__ __forceinline__ bool exchange_cell(double r, double& t, double& er, const Opacity& op,
                                               double dtc, double a_r, double cv) {
     if (!(pos_finite(r) && pos_finite(t) && pos_finite(er))) return false;
-    const double kap = opacity_eval<kTables>(op, r, t);
-    if (!pos_finite(kap)) return false;
-    exchange_cell_kr(r, kap * r, t, er, dtc, a_r, cv);
+    double kr;
+    if (!kapparho<kTables>(op, r, t, kr)) return false;
+    exchange_cell_kr(r, kr, t, er, dtc, a_r, cv);
     return true;
 }
 

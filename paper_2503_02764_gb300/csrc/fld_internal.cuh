@@ -133,28 +133,6 @@ __device__ __forceinline__ double rcp_nr(double a) {
     return fma(y, e, y);
 }
 
-// n / d for n >= 0 and 0 < d within the FP32 normal range (and 1/d too): one Newton-
-// Raphson step on the FP32 reciprocal, the quotient, and one correction from its exact
-// remainder n - d q (Markstein's scheme): within a unit of rounding, five FP64 operations.
-__device__ __forceinline__ double div_nr(double n, double d) {
-    double y = f64_of_pos(__frcp_rn(f32_near_pos(d)));
-    y = fma(y, fma(-d, y, 1.0), y);
-    const double q = n * y;
-    return fma(fma(-d, q, n), y, q);
-}
-
-// sqrt(t) for 0 < t within the FP32 normal range: from the FP32 reciprocal square root
-// y0, s = t y0 corrected twice by s <- s + (t - s^2) y0 / 2 (a Newton step for s^2 = t
-// with the derivative's inverse taken from the seed): relative error 1.5 e0^2 after the
-// first, rounding after the second; five FP64 operations.
-__device__ __forceinline__ double sqrt_nr(double t) {
-    const float y0 = rsqrtf(f32_near_pos(t));
-    const double hy = f64_of_pos(0.5f * y0);
-    double s = t * f64_of_pos(y0);
-    s = fma(fma(-s, s, t), hy, s);
-    return fma(fma(-s, s, t), hy, s);
-}
-
 // |v| within [2^-99, 2^99] (safely inside the FP32 normal range), tested on the
 // exponent bits with integer operations.
 __device__ __forceinline__ bool in_f32_range(double v) {

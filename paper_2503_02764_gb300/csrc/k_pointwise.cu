@@ -24,7 +24,7 @@ namespace fld {
 // kr (nullable): kappa rho of every cell, frozen at the step's start by the limiter of the
 // same substep; without it kappa is evaluated from (rho, T). DF as for k_limiter.
 template <bool DF>
-__global__ void __launch_bounds__(256, DF ? 5 : 6) k_exchange(long long n, const double* __restrict__ rho, double* __restrict__ T,
+__global__ void __launch_bounds__(256, 5) k_exchange(long long n, const double* __restrict__ rho, double* __restrict__ T,
                            double* __restrict__ E, const double* __restrict__ kr, Opacity op,
                            double dtc, double a_r, double cv, int use_df, DfConst K,
                            unsigned* err, double one) {
@@ -97,11 +97,26 @@ __global__ void k_split_df(long long n, const double* __restrict__ v, float* __r
     }
 }
 
+// The FP64 routine of the cells that the double-FP32 one declines, out of line: its registers
+// would cost the double-FP32 kernel its fifth block per SM.
+static __device__ __noinline__ bool limiter_cell_64(const Lvl& L, const double* ih, const double* E,
+                                                    const double* rho, const double* T,
+                                                    const double* Ebc, const BcOff& bo,
+                                                    const Opacity& op, double c, int mode, int i,
+                                                    int j, int k, long long p, double& D,
+                                                    double& lm, double* kr) {
+    return limiter_cell(L, ih, E, rho, T, Ebc, bo, op, c, mode, i, j, k, p, D, lm, kr);
+}
+
+struct Df3 {             // 1/(12 h_d) as pairs, split once on the host
+    df v[3];
+};
+
 // kr (nullable): receives kappa rho of every cell, for the exchange of the same substep.
 // DF: the double-FP32 cell routine first (FP64 for the cells it declines); the FP64-only
 // instantiation carries none of its registers.
 template <bool DF>
-__global__ void __launch_bounds__(256, DF ? 5 : 6) k_limiter(Lvl L, double3 inv12h, const double* __restrict__ E,
+__global__ void __launch_bounds__(256, DF ? 5 : 4) k_limiter(Lvl L, double3 inv12h, Df3 inv12hd, const double* __restrict__ E,
                           const double* __restrict__ rho, const double* __restrict__ T,
                           const double* __restrict__ Ebc, BcOff bo, Opacity op, double c,
                           int mode, int use_df, DfConst K, const float* __restrict__ Eh,
@@ -109,14 +124,13 @@ __global__ void __launch_bounds__(256, DF ? 5 : 6) k_limiter(Lvl L, double3 inv1
                           double* __restrict__ lam, double* __restrict__ kr, unsigned* err,
                           double one) {
     const double ih[3] = {inv12h.x, inv12h.y, inv12h.z};
-    df ihd[3];
-    if (DF)
-        for (int d = 0; d < 3; ++d) ihd[d] = df_from_double(ih[d]);
-    const int nrows = L.n[1] * L.n[2];
-    for (int rw = blockIdx.x; rw < nrows; rw += gridDim.x)
-        for (int i = threadIdx.x; i < L.n[0]; i += blockDim.x) {
-            const int j = rw % L.n[1], k = rw / L.n[1];
-            const long long p = (long long)rw * L.n[0] + i;
+    const df ihd[3] = {inv12hd.v[0], inv12hd.v[1], inv12hd.v[2]};
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= L.n[0]) return;
+    for (int k = blockIdx.z; k < L.n[2]; k += gridDim.z)
+        for (int j = blockIdx.y * blockDim.y + threadIdx.y; j < L.n[1];
+             j += gridDim.y * blockDim.y) {
+            const long long p = ((long long)k * L.n[1] + j) * L.n[0] + i;
             double Dv, lm, kv;
             if (DF && use_df && limiter_cell_df(L, ih, E, rho, T, Ebc, bo, op, K, mode, i, j, k, p, Dv, lm,
                                           Eh, El, ihd, kr ? &kv : nullptr)) {
@@ -125,8 +139,10 @@ __global__ void __launch_bounds__(256, DF ? 5 : 6) k_limiter(Lvl L, double3 inv1
                 if (kr) kr[p] = kv;
                 continue;
             }
-            if (!limiter_cell(L, ih, E, rho, T, Ebc, bo, op, c, mode, i, j, k, p, Dv, lm,
-                              kr ? &kv : nullptr, lam != nullptr, one)) {
+            if (!(DF ? limiter_cell_64(L, ih, E, rho, T, Ebc, bo, op, c, mode, i, j, k, p, Dv, lm,
+                                       &kv)
+                     : limiter_cell(L, ih, E, rho, T, Ebc, bo, op, c, mode, i, j, k, p, Dv, lm,
+                                    kr ? &kv : nullptr, lam != nullptr, one))) {
                 atomicOr(err, ERRBIT_DOMAIN);
                 continue;
             }
@@ -137,67 +153,78 @@ __global__ void __launch_bounds__(256, DF ? 5 : 6) k_limiter(Lvl L, double3 inv1
 }
 
 // ----------------------------------------------------------------- coupling terms
-// v_c at offset o (|o| <= 2) along axis d: periodic wrap, an even mirror at walls.
-__device__ __forceinline__ double fetch_v(const Lvl& L, const double* __restrict__ v, int i,
-                                          int j, int k, int d, int o) {
-    int c[3] = {i, j, k};
-    const int n = L.n[d];
-    int m = c[d] + o;
-    if (m < 0) m = L.bclo[d] == FLD_BC_PERIODIC ? m + n : -m - 1;
-    else if (m >= n) m = L.bchi[d] == FLD_BC_PERIODIC ? m - n : 2 * n - 1 - m;
-    c[d] = m;
-    return v[lin(L, c[0], c[1], c[2])];
+// v_-2, v_-1, v_+1, v_+2 along axis d: periodic wrap, an even mirror at walls.
+__device__ __forceinline__ void fetch_v(const Lvl& L, const double* __restrict__ v, int c, int d,
+                                        int p, double w[4]) {
+    const int n = L.n[d], st = d == 0 ? 1 : d == 1 ? L.n[0] : L.n[0] * L.n[1];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        int m = c + (q < 2 ? q - 2 : q - 1);
+        if (m < 0) m = L.bclo[d] == FLD_BC_PERIODIC ? m + n : -m - 1;
+        else if (m >= n) m = L.bchi[d] == FLD_BC_PERIODIC ? m - n : 2 * n - 1 - m;
+        w[q] = v[p + (m - c) * st];
+    }
 }
 
 // Explicit coupling terms of one cell, in FP64 from the limiter's gradient: F = -D grad E,
 // f_r = -lambda grad E, f = lambda + lambda^2 R^2, and with v: v . f_r and
-// P : grad v, P = E ((1 - f) I + (3f - 1) n n) / 2, n = grad E / |grad E|.
-__global__ void k_coupling(Lvl L, double3 inv12h, double3 inv12hv, const double* __restrict__ E,
-                           const double* __restrict__ rho, const double* __restrict__ T,
-                           const double* __restrict__ Ebc, BcOff bo, Opacity op, double c,
-                           int mode, const double* __restrict__ v, double* __restrict__ F,
-                           double* __restrict__ fr, double* __restrict__ fe,
-                           double* __restrict__ vfr, double* __restrict__ pt, unsigned* err) {
+// P : grad v, P = E ((1 - f) I + (3f - 1) n n) / 2, n = grad E / |grad E|, contracted as
+//   E ((1 - f)/2 div v + (3f - 1)/(2 g^2) sum_ij g_i g_j d_j v_i).
+// FP64 issue bounds it (88 % of the pipe with IEEE divisions and roots and the twelve
+// differences in FP64, 166 instructions a cell): lambda / a is one fix_div as in the limiter,
+// lambda R = g (lambda / a), and the differences run in fixed point (fix64.cuh).
+__global__ void __launch_bounds__(256, 3)
+k_coupling(Lvl L, double3 inv12h, const double* __restrict__ E,
+           const double* __restrict__ rho, const double* __restrict__ T,
+           const double* __restrict__ Ebc, BcOff bo, Opacity op, double c,
+           int mode, const double* __restrict__ v, double* __restrict__ F,
+           double* __restrict__ fr, double* __restrict__ fe,
+           double* __restrict__ vfr, double* __restrict__ pt, unsigned* err, double one) {
     const double ih[3] = {inv12h.x, inv12h.y, inv12h.z};
-    const double ihv[3] = {inv12hv.x, inv12hv.y, inv12hv.z};
-    const int nd = L.ndim;
     const long long nc = L.ncell;
-    const int nrows = L.n[1] * L.n[2];
-    for (int rw = blockIdx.x; rw < nrows; rw += gridDim.x)
-        for (int i = threadIdx.x; i < L.n[0]; i += blockDim.x) {
-            const int j = rw % L.n[1], k = rw / L.n[1];
-            const long long p = (long long)rw * L.n[0] + i;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= L.n[0]) return;
+    for (int k = blockIdx.z; k < L.n[2]; k += gridDim.z)
+        for (int j = blockIdx.y * blockDim.y + threadIdx.y; j < L.n[1];
+             j += gridDim.y * blockDim.y) {
+            const int p = (k * L.n[1] + j) * L.n[0] + i;
             const double Ec = E[p], r = rho[p];
             const double t = op.kind == FLD_OPACITY_CONST ? 1.0 : T[p];
-            if (!(pos_finite(Ec) && pos_finite(r) && pos_finite(t))) {
-                atomicOr(err, ERRBIT_DOMAIN);
-                continue;
-            }
-            const double kap = opacity_eval(op, r, t);
-            if (!pos_finite(kap)) {
+            double kr;
+            if (!(pos_finite(Ec) && pos_finite(r) && pos_finite(t)) ||
+                !kapparho<true>(op, r, t, kr)) {
                 atomicOr(err, ERRBIT_DOMAIN);
                 continue;
             }
             double g[3] = {0.0, 0.0, 0.0};
             double g2 = 0.0;
-            for (int d = 0; d < nd; ++d) {
-                const double em2 = fetch_E(L, E, Ebc, bo, i, j, k, d, -2);
-                const double em1 = fetch_E(L, E, Ebc, bo, i, j, k, d, -1);
-                const double ep1 = fetch_E(L, E, Ebc, bo, i, j, k, d, 1);
-                const double ep2 = fetch_E(L, E, Ebc, bo, i, j, k, d, 2);
-                g[d] = ((em2 - 8.0 * em1) + 8.0 * ep1 - ep2) * ih[d];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                if (d >= L.ndim) break;
+                double w[4];
+                fetch_axis(L, E, Ebc, bo, i, j, k, d, p, w);
+                g[d] = fix_stencil(w[0], w[1], w[2], w[3]) * ih[d];
                 g2 = fma(g[d], g[d], g2);
             }
-            const double gn = sqrt(g2);
-            const double kr = kap * r;
-            const double R = gn / (kr * Ec);
-            const double lam = mode == FLD_LIMITER_LP        ? (2.0 + R) / (6.0 + 3.0 * R + R * R)
-                               : mode == FLD_LIMITER_MINERBO ? minerbo_lambda(R)
-                                                             : 1.0 / 3.0;
-            const double D = c * lam / kr;
-            const double f = lam + lam * lam * R * R;
+            const double a = kr * Ec;
+            double lam, lr, D, gn, q;          // lr = lambda R
+            if (mode != FLD_LIMITER_DIFFUSION && limiter_core<true>(a, g2, mode, one, true, gn, q, lam)) {
+                lr = gn * q;
+                D = c * Ec * q;
+            } else {
+                gn = sqrt(g2);
+                const double R = gn / a;
+                lam = mode == FLD_LIMITER_LP        ? (2.0 + R) / (6.0 + 3.0 * R + R * R)
+                      : mode == FLD_LIMITER_MINERBO ? minerbo_lambda(R)
+                                                    : 1.0 / 3.0;
+                lr = lam * R;
+                D = c * lam / kr;
+            }
+            const double f = fma(lr, lr, lam);
             double vf = 0.0;
-            for (int d = 0; d < nd; ++d) {
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                if (d >= L.ndim) break;
                 const double frd = -lam * g[d];
                 if (F) F[d * nc + p] = -D * g[d];
                 if (fr) fr[d * nc + p] = frd;
@@ -206,25 +233,41 @@ __global__ void k_coupling(Lvl L, double3 inv12h, double3 inv12hv, const double*
             if (fe) fe[p] = f;
             if (v && vfr) vfr[p] = vf;
             if (v && pt) {
-                double n[3] = {0.0, 0.0, 0.0};
-                if (gn > 0.0)
-                    for (int d = 0; d < nd; ++d) n[d] = g[d] / gn;
-                const double a = 0.5 * (1.0 - f), bq = 0.5 * (3.0 * f - 1.0);
-                double acc = 0.0;
-                for (int a1 = 0; a1 < nd; ++a1) {            // velocity component
+                double gh[3], div = 0.0, S = 0.0;
+                const int cc[3] = {i, j, k};
+#pragma unroll
+                for (int d = 0; d < 3; ++d) gh[d] = d < L.ndim ? g[d] * ih[d] : 0.0;
+#pragma unroll
+                for (int a1 = 0; a1 < 3; ++a1) {             // velocity component
+                    if (a1 >= L.ndim) break;
                     const double* vi = v + a1 * nc;
-                    for (int a2 = 0; a2 < nd; ++a2) {        // derivative axis
-                        const double gv = ((fetch_v(L, vi, i, j, k, a2, -2) -
-                                            8.0 * fetch_v(L, vi, i, j, k, a2, -1)) +
-                                           8.0 * fetch_v(L, vi, i, j, k, a2, 1) -
-                                           fetch_v(L, vi, i, j, k, a2, 2)) * ihv[a2];
-                        const double Pij = ((a1 == a2 ? a : 0.0) + bq * n[a1] * n[a2]) * Ec;
-                        acc = fma(Pij, gv, acc);
+                    double gv = 0.0;
+#pragma unroll
+                    for (int a2 = 0; a2 < 3; ++a2) {         // derivative axis
+                        if (a2 >= L.ndim) break;
+                        double w[4];
+                        fetch_v(L, vi, cc[a2], a2, p, w);
+                        const double s = fix_stencil(w[0], w[1], w[2], w[3]);
+                        gv = fma(gh[a2], s, gv);
+                        if (a1 == a2) div = fma(ih[a2], s, div);
                     }
+                    S = fma(g[a1], gv, S);
                 }
-                pt[p] = acc;
+                double acc = 0.5 * fma(f, -one, 1.0) * div;
+                if (gn > 0.0) {
+                    const double bq = fma(1.5, f, -0.5);
+                    acc = fma(div_ok(1.0, g2) ? bq * fix_div(1.0, g2) : bq / g2, S, acc);
+                }
+                pt[p] = Ec * acc;
             }
         }
+}
+
+// blocks of 32 x 8 cells, or of a line's cells in a row
+static dim3 cell_block(const Lvl& L) { return L.n[1] > 1 ? dim3(32, 8) : dim3(256, 1); }
+static dim3 cell_grid(const Lvl& L, dim3 blk) {
+    return dim3((L.n[0] + blk.x - 1) / blk.x, std::min<int>((L.n[1] + blk.y - 1) / blk.y, 65535),
+                std::min(L.n[2], 65535));
 }
 
 void launch_coupling(const Lvl& L, const double* h, const double* E, const double* rho,
@@ -235,9 +278,9 @@ void launch_coupling(const Lvl& L, const double* h, const double* E, const doubl
     for (int q = 0; q < 6; ++q) bo.off[q] = bc_off[q];
     const double3 ih = make_double3(1.0 / (12.0 * h[0]), L.ndim > 1 ? 1.0 / (12.0 * h[1]) : 0.0,
                                     L.ndim > 2 ? 1.0 / (12.0 * h[2]) : 0.0);
-    const int nb = (int)std::min<long long>((long long)L.n[1] * L.n[2], num_sms() * 64);
-    k_coupling<<<nb, 256, 0, s>>>(L, ih, ih, E, rho, T, E_bc, bo, op, c, mode, v, F, fr, fe, vfr,
-                                  pt, err);
+    const dim3 blk = cell_block(L);
+    k_coupling<<<cell_grid(L, blk), blk, 0, s>>>(L, ih, E, rho, T, E_bc, bo, op, c, mode, v, F,
+                                                 fr, fe, vfr, pt, err, 1.0);
 }
 
 void launch_split_df(long long n, const double* v, float* hi, float* lo, cudaStream_t s) {
@@ -253,15 +296,18 @@ void launch_limiter(const Lvl& L, const double* h, const double* E, const double
     for (int q = 0; q < 6; ++q) bo.off[q] = bc_off[q];
     double3 ih = make_double3(1.0 / (12.0 * h[0]), L.ndim > 1 ? 1.0 / (12.0 * h[1]) : 0.0,
                               L.ndim > 2 ? 1.0 / (12.0 * h[2]) : 0.0);
-    const int block = 256;
-    const int nb = (int)std::min<long long>((long long)L.n[1] * L.n[2], num_sms() * 64);
+    const dim3 block = cell_block(L), nb = cell_grid(L, block);
     const DfConst K = make_dfconst(c, op.kappa0, 0.0, 0.0, 0.0);
+    Df3 ihd;
+    split_host(ih.x, ihd.v[0].hi, ihd.v[0].lo);
+    split_host(ih.y, ihd.v[1].hi, ihd.v[1].lo);
+    split_host(ih.z, ihd.v[2].hi, ihd.v[2].lo);
     if (!(use_df && mode != FLD_LIMITER_DIFFUSION)) Eh = El = nullptr;
     if (use_df)
-        k_limiter<true><<<nb, block, 0, s>>>(L, ih, E, rho, T, E_bc, bo, op, c, mode, use_df, K,
+        k_limiter<true><<<nb, block, 0, s>>>(L, ih, ihd, E, rho, T, E_bc, bo, op, c, mode, use_df, K,
                                              Eh, El, D, lam, kr, err, 1.0);
     else
-        k_limiter<false><<<nb, block, 0, s>>>(L, ih, E, rho, T, E_bc, bo, op, c, mode, use_df, K,
+        k_limiter<false><<<nb, block, 0, s>>>(L, ih, ihd, E, rho, T, E_bc, bo, op, c, mode, use_df, K,
                                               Eh, El, D, lam, kr, err, 1.0);
 }
 
