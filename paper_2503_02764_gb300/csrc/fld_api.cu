@@ -508,9 +508,25 @@ void smooth(fld_handle* h, LevelBufs<T>& B, int l, int n, int fused, T*& cur, T*
     }
 }
 
-// -------------------------------------------------- V-cycle on level l (x_l in/out)
+// 2D FP32 levels whose two sides run as one launch each
 template <typename T>
-void vcycle(fld_handle* h, LevelBufs<T>* P, int l, cudaStream_t s) {
+bool tile_level(const fld_handle* h, int l) {
+    if (sizeof(T) != 4 || h->o.smoother == 1 || l == h->nlev - 1) return false;
+    if (l == h->vdepth - 1) return tile2d_ok(h->lv[l], h->vsweeps);
+    return l != h->tail_start && tile2d_ok(h->lv[l], std::max(h->o.nu1, h->o.nu2));
+}
+
+// the starting iterate of level l, where the V-cycle reads it
+template <typename T>
+void zero_level(fld_handle* h, LevelBufs<T>* P, int l, cudaStream_t s) {
+    if (l < h->nlev - 1 && !tile_level<T>(h, l))
+        cudaMemsetAsync(P[l].x, 0, sizeof(T) * h->lv[l].ncell, s);
+}
+
+// -------------------------------------------------- V-cycle on level l (x_l in/out; with
+// `zero` the iterate starts from zero: a tile level then reads no x_l, the others find zeros)
+template <typename T>
+void vcycle(fld_handle* h, LevelBufs<T>* P, int l, bool zero, cudaStream_t s) {
     const Lvl& L = h->lv[l];
     LevelBufs<T>& B = P[l];
     const bool f32 = sizeof(T) == 4;
@@ -519,13 +535,34 @@ void vcycle(fld_handle* h, LevelBufs<T>* P, int l, cudaStream_t s) {
             [&] { launch_coarse_solve<T>(L, B.x, B.b, B.K, h->o.coarse_sweeps, s); });
         return;
     }
+    if constexpr (sizeof(T) == 4) {
+        if (tile_level<T>(h, l)) {
+            if (l == h->vdepth - 1) {
+                run(h, "tile32", l, L.ncell, s, [&] {
+                    launch_tile2d(L, L, nullptr, B.x, B.b, B.K, nullptr, nullptr, h->vsweeps, s);
+                });
+                return;
+            }
+            LevelBufs<T>& Cb = P[l + 1];
+            run(h, "tile32", l, L.ncell, s, [&] {
+                launch_tile2d(L, h->lv[l + 1], zero ? nullptr : B.x, B.tmp, B.b, B.K, nullptr, Cb.b,
+                              h->o.nu1, s);
+            });
+            zero_level<T>(h, P, l + 1, s);
+            vcycle<T>(h, P, l + 1, true, s);
+            run(h, "tile32", l, L.ncell, s, [&] {
+                launch_tile2d(L, h->lv[l + 1], B.tmp, B.x, B.b, B.K, Cb.x, nullptr, h->o.nu2, s);
+            });
+            return;
+        }
+    }
     if (l == h->vdepth - 1) {
         // the truncated coarsest level: vsweeps red-black sweeps from x = 0 (an even
         // number of them single-pass, so the iterate ends in B.x)
         T* cur = B.x;
         T* oth = B.tmp;
         const int n = h->vsweeps;
-        const int f = (h->o.smoother == 2 && rb_sweep_supported<T>(L)) ? (n & ~1) : 0;
+        const int f = (h->o.smoother != 1 && rb_sweep_supported<T>(L)) ? (n & ~1) : 0;
         smooth<T>(h, B, l, n, f, cur, oth, s);
         return;
     }
@@ -550,7 +587,7 @@ void vcycle(fld_handle* h, LevelBufs<T>* P, int l, cudaStream_t s) {
     // to B.x; with an odd nu1 + nu2 the last sweep of the cycle runs in place
     const int nu1 = h->o.nu1, nu2 = h->o.nu2;
     int f1 = 0, f2 = 0;
-    if (h->o.smoother == 2 && rb_sweep_supported<T>(L)) {
+    if (h->o.smoother != 1 && rb_sweep_supported<T>(L)) {
         f1 = nu1;
         f2 = nu2;
         if ((nu1 + nu2) & 1) (nu2 > 0 ? f2 : f1) -= 1;
@@ -567,8 +604,8 @@ void vcycle(fld_handle* h, LevelBufs<T>* P, int l, cudaStream_t s) {
         }
         launch_resid_restrict<T>(L, C, cur, B.b, B.K, P[l + 1].b, bs, nu1 > 0, s);
     });
-    if (l + 1 < h->nlev - 1) cudaMemsetAsync(P[l + 1].x, 0, sizeof(T) * C.ncell, s);
-    vcycle<T>(h, P, l + 1, s);
+    zero_level<T>(h, P, l + 1, s);
+    vcycle<T>(h, P, l + 1, true, s);
     run(h, f32 ? "prolong32" : "prolong64", l, L.ncell, s,
         [&] { launch_prolong<T>(L, C, cur, P[l + 1].x, bs, s); });
     smooth<T>(h, B, l, nu2, f2, cur, oth, s);
@@ -601,7 +638,7 @@ fld_status read_scalars(fld_handle* h, cudaStream_t s, double* sum, unsigned* er
 }
 
 // relative residual of x at level 0 (FP64), optional FP32 copy of the residual. With e
-// (3D levels, where the z-marching kernel applies) the iterate is first corrected: x + e is
+// (2D and 3D levels with the arithmetic face mean) the iterate is first corrected: x + e is
 // written to xo and the residual is that of xo.
 fld_status residual(fld_handle* h, const double* x, const float* e, double* xo, float* r32,
                     cudaStream_t s, double* rr, unsigned* err) {
@@ -616,6 +653,11 @@ fld_status residual(fld_handle* h, const double* x, const float* e, double* xo, 
         run(h, e ? "resid64x" : "resid64", 0, L.ncell, s, [&] {
             nparts = launch_resid64z(L, x, e, xo, h->d64[0].b, h->d64[0].K, r32, h->partials,
                                      h->norm_blocks, s);
+        });
+    } else if (resid64_2d_ok(L)) {
+        run(h, e ? "resid64x" : "resid64", 0, L.ncell, s, [&] {
+            nparts = launch_resid64_2d(L, x, e, xo, h->d64[0].b, h->d64[0].K, r32, h->partials,
+                                       h->norm_blocks, s);
         });
     } else {
         run(h, "resid64", 0, L.ncell, s, [&] {
@@ -675,8 +717,9 @@ fld_status vcycle32(fld_handle* h, cudaStream_t s) {
     const long long n0 = h->lv[0].ncell;
     const int inner = h->o.inner > 0 ? h->o.inner : 1;
     if (!h->o.graph || h->prof.on) {
-        FLD_CK(cudaMemsetAsync(h->d32[0].x, 0, sizeof(float) * n0, s));
-        for (int c = 0; c < inner; ++c) vcycle<float>(h, h->d32, 0, s);
+        if (!tile_level<float>(h, 0))
+            FLD_CK(cudaMemsetAsync(h->d32[0].x, 0, sizeof(float) * n0, s));
+        for (int c = 0; c < inner; ++c) vcycle<float>(h, h->d32, 0, c == 0, s);
         return FLD_OK;
     }
     const int key[8] = {h->o.nu1, h->o.nu2, h->o.smoother, h->o.block, h->o.coarse_sweeps,
@@ -692,8 +735,9 @@ fld_status vcycle32(fld_handle* h, cudaStream_t s) {
         cudaGraph_t g = nullptr;
         const long long before = g_launches.load();
         FLD_CK(cudaStreamBeginCapture(h->gs, cudaStreamCaptureModeThreadLocal));
-        cudaMemsetAsync(h->d32[0].x, 0, sizeof(float) * n0, h->gs);
-        for (int c = 0; c < inner; ++c) vcycle<float>(h, h->d32, 0, h->gs);
+        if (!tile_level<float>(h, 0))
+            cudaMemsetAsync(h->d32[0].x, 0, sizeof(float) * n0, h->gs);
+        for (int c = 0; c < inner; ++c) vcycle<float>(h, h->d32, 0, c == 0, h->gs);
         FLD_CK(cudaStreamEndCapture(h->gs, &g));
         h->vgraph_nodes = g_launches.load() - before;
         g_launches.fetch_sub(h->vgraph_nodes);       // counted per replay below
@@ -971,10 +1015,10 @@ fld_status diffuse_impl(fld_handle* h, double dt, const double* D, const double*
         st->resid_hist[0] = rel;
         st->levels = h->vdepth;
     }
-    // mixed refinement on 3D levels: the correction is added inside the residual kernel,
+    // mixed refinement on 2D and 3D levels: the correction is added inside the residual kernel,
     // out of place, the iterate alternating between E and the level-0 FP64 scratch (free
     // in this mode); it ends in E
-    const bool fused = mixed && resid64z_ok(L0, h->norm_blocks);
+    const bool fused = mixed && (resid64z_ok(L0, h->norm_blocks) || resid64_2d_ok(L0));
     // after the first FP64 residual, the later ones may be updated recursively (r - A e in
     // FP32) while the accumulated rounding bound `drift` stays below tol/2 ||b||; the scale
     // of the squared sums is 2^-k with 2^k near the RMS of b
@@ -1021,7 +1065,7 @@ fld_status diffuse_impl(fld_handle* h, double dt, const double* D, const double*
                 [&] { launch_add_correction(L0.ncell, E, h->d32[0].x, s); });
             rc = residual(h, E, nullptr, nullptr, h->d32[0].b, s, &r2, &err);
         } else {
-            vcycle<double>(h, h->d64, 0, s);
+            vcycle<double>(h, h->d64, 0, false, s);
             rc = residual(h, E, nullptr, nullptr, nullptr, s, &r2, &err);
         }
         if (rc != FLD_OK) break;
@@ -1129,6 +1173,7 @@ fld_status fld_create(fld_handle** out, const fld_grid* g, const fld_opts* o) {
         prepare_rb_sweep();
         prepare_vcycle_tail();
         prepare_line();
+        prepare_tile2d();
         debug_attach_all();
     }
     if (!rc && cudaDeviceSynchronize() != cudaSuccess) rc = FLD_ERR_CUDA;
@@ -1396,7 +1441,7 @@ fld_status fld::fld_correction(fld_handle* h, const double* r, double* e, int cy
         FLD_CK(cudaMemcpyAsync(h->d64[0].b, r, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
         FLD_CK(cudaMemsetAsync(e, 0, sizeof(double) * n, s));
         h->d64[0].x = e;
-        for (int c = 0; c < cycles; ++c) vcycle<double>(h, h->d64, 0, s);
+        for (int c = 0; c < cycles; ++c) vcycle<double>(h, h->d64, 0, false, s);
     } else {
         run(h, "to_f32", 0, n, s, [&] { launch_to_f32(n, r, h->d32[0].b, s); });
         const int inner = h->o.inner;
@@ -1567,6 +1612,7 @@ extern "C" fld_status fld_diffuse_static(const fld_grid* g, const fld_opts* o, d
     h.o.direct1d = 0;     // V-cycles in every dimension (the workspace holds no direct solver)
     prepare_rb_sweep();   // kernel attributes only (no device memory)
     prepare_vcycle_tail();
+    prepare_tile2d();
     build_levels(&h);
     h.ncell = h.lv[0].ncell;
     long long off = 0;

@@ -244,6 +244,14 @@ bool rb_sweep_supported(const Lvl& L);
 template <typename T>
 void launch_rb_sweep(const Lvl& L, const T* xin, T* xout, const T* b, const T* K, cudaStream_t s);
 void prepare_rb_sweep();
+// One side of a 2D FP32 level in one launch (k_tile2d.cu): xout = `sweeps` red-black sweeps of
+// xin (null: zero; ec non-null: plus the prolonged coarse correction), and with bc non-null the
+// restricted residual of xout. xout is not xin.
+constexpr int TILE2D_SWEEPS = 4;
+bool tile2d_ok(const Lvl& L, int sweeps);
+void prepare_tile2d();
+void launch_tile2d(const Lvl& F, const Lvl& C, const float* xin, float* xout, const float* b,
+                   const float* K, const float* ec, float* bc, int sweeps, cudaStream_t s);
 // The coarse end of a V-cycle in one single-block launch: the levels from the first with at
 // most TAIL_MAX_CELLS cells to the coarsest (which must hold at most TAIL_MAX_DENSE cells).
 constexpr long long TAIL_MAX_CELLS = 512;
@@ -322,6 +330,10 @@ bool resid64z_ok(const Lvl& L, int nblocks);
 // block per row; returns the number of partial sums written (<= nblocks)
 int launch_resid32_init(const Lvl& L, const double* x, const double* b, const float* K,
                         float* r32, double* partials, int nblocks, cudaStream_t s);
+// the same on 2D levels with the arithmetic face mean
+bool resid64_2d_ok(const Lvl& L);
+int launch_resid64_2d(const Lvl& L, const double* x, const float* e, double* xo, const double* b,
+                      const double* K, float* r32, double* partials, int nblocks, cudaStream_t s);
 int launch_resid64z(const Lvl& L, const double* x, const float* e, double* xo, const double* b,
                     const double* K, float* r32, double* partials, int nblocks, cudaStream_t s);
 // Recursive refinement residual (k_resupd.cu): xo = x + e, r32 <- r32 - A e in FP32 on the

@@ -239,6 +239,71 @@ k_resid64z(Lvl L, const double* __restrict__ x, const float* __restrict__ e,
     if (threadIdx.x == 0) partials[blockIdx.x] = a2;
 }
 
+// The same on a 2D level: tiles of 32 x 8 cells with a one-cell ring, two fluxes a cell. The
+// kernel it replaced there evaluated four (one block a row, 50 us at 1024^2 beside a launch of
+// its own for x + e).
+__global__ void __launch_bounds__(RZ_NT)
+k_resid64_2d(Lvl L, const double* __restrict__ x, const float* __restrict__ e,
+             double* __restrict__ xo, const double* __restrict__ b, const double* __restrict__ K,
+             float* __restrict__ r32, double* __restrict__ partials, double one) {
+    __shared__ double XS[(RZ_TY + 2) * RZ_PW], KS[(RZ_TY + 2) * RZ_PW];
+    __shared__ double FX[RZ_TY * (RZ_TX + 1)], FY[(RZ_TY + 1) * RZ_TX];
+    __shared__ double sh[32];
+    const int nx = L.n[0], ny = L.n[1];
+    const int tilesx = (nx + RZ_TX - 1) / RZ_TX, tiles = tilesx * ((ny + RZ_TY - 1) / RZ_TY);
+    const bool xper = L.bclo[0] == FLD_BC_PERIODIC, yper = L.bclo[1] == FLD_BC_PERIODIC;
+    const double hx = 0.5 * L.w[0], hy = 0.5 * L.w[1];
+    const int tid = threadIdx.x, lx = tid % RZ_TX, ly = tid / RZ_TX;
+    double acc2 = 0.0;
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int tx0 = (t % tilesx) * RZ_TX, ty0 = (t / tilesx) * RZ_TY;
+        const int ax = min(RZ_TX, nx - tx0), ay = min(RZ_TY, ny - ty0);
+        for (int q = tid; q < (ay + 2) * (ax + 2); q += RZ_NT) {
+            const int qy = q / (ax + 2) - 1, qx = q - (qy + 1) * (ax + 2) - 1;
+            const int gx = rz_axis(tx0 + qx, nx, xper), gy = rz_axis(ty0 + qy, ny, yper);
+            const int so = (qy + 1) * RZ_PW + qx + 1;
+            if (gx >= 0 && gy >= 0) {
+                const int p = (int)fld_at((long long)gy * nx + gx, L.ncell);
+                const double v = e ? addf(x[p], f64_of(e[p]), one) : x[p];
+                XS[so] = v;
+                KS[so] = K[p];
+                if (xo && qx >= 0 && qx < ax && qy >= 0 && qy < ay) xo[p] = v;
+            } else if (gx >= 0 || gy >= 0) {     // a wall ghost (corners are not read)
+                const int wx = gx >= 0 ? gx : (qx < 0 ? 0 : nx - 1);
+                const int wy = gy >= 0 ? gy : (qy < 0 ? 0 : ny - 1);
+                const int bc = gx < 0 ? (qx < 0 ? L.bclo[0] : L.bchi[0])
+                                      : (qy < 0 ? L.bclo[1] : L.bchi[1]);
+                XS[so] = 0.0;
+                KS[so] = rz_factor(bc) * K[(long long)wy * nx + wx];
+            }
+        }
+        __syncthreads();
+        const bool act = lx < ax && ly < ay;
+        const int so = (ly + 1) * RZ_PW + lx + 1;
+        auto flux = [&](int c, int q) {
+            return addf(KS[c], KS[q], one) * subf(XS[c], XS[q], one);
+        };
+        if (act) {
+            FX[ly * (RZ_TX + 1) + lx] = flux(so, so - 1);
+            if (lx == ax - 1) FX[ly * (RZ_TX + 1) + lx + 1] = flux(so + 1, so);
+            FY[ly * RZ_TX + lx] = flux(so, so - RZ_PW);
+            if (ly == ay - 1) FY[(ly + 1) * RZ_TX + lx] = flux(so + RZ_PW, so);
+        }
+        __syncthreads();
+        if (act) {
+            const int p = (ty0 + ly) * nx + tx0 + lx;
+            const int fx = ly * (RZ_TX + 1) + lx, fy = ly * RZ_TX + lx;
+            double r = fma(-hx, subf(FX[fx], FX[fx + 1], one), subf(b[p], XS[so], one));
+            r = fma(-hy, subf(FY[fy], FY[fy + RZ_TX], one), r);
+            if (r32) r32[p] = f32_of(r);
+            acc2 = fma(r, r, acc2);
+        }
+        __syncthreads();
+    }
+    const double a2 = block_sum(acc2, sh);
+    if (threadIdx.x == 0) partials[blockIdx.x] = a2;
+}
+
 int g_rz_slots[64];        // resident blocks of the kernel on the whole GPU, per device
 
 }  // namespace
@@ -247,6 +312,17 @@ bool resid64z_ok(const Lvl& L, int nblocks) {
     if (L.ndim != 3 || L.fm) return false;     // arithmetic face mean only
     const int tiles = ((L.n[0] + RZ_TX - 1) / RZ_TX) * ((L.n[1] + RZ_TY - 1) / RZ_TY);
     return tiles <= nblocks;
+}
+
+bool resid64_2d_ok(const Lvl& L) { return L.ndim == 2 && !L.fm; }
+
+int launch_resid64_2d(const Lvl& L, const double* x, const float* e, double* xo, const double* b,
+                      const double* K, float* r32, double* partials, int nblocks, cudaStream_t s) {
+    const long long tiles = (long long)((L.n[0] + RZ_TX - 1) / RZ_TX) *
+                            ((L.n[1] + RZ_TY - 1) / RZ_TY);
+    const int nb = (int)std::min<long long>(tiles, nblocks);
+    k_resid64_2d<<<nb, RZ_NT, 0, s>>>(L, x, e, xo, b, K, r32, partials, 1.0);
+    return nb;
 }
 
 // Returns the number of partial sums written (the blocks of the launch, <= nblocks).
