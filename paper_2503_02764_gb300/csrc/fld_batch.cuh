@@ -44,7 +44,7 @@ struct BatchStat {
 int batch_threads_supported(int nt);
 int batch_cluster_supported(int cs);
 // groups (clusters of cs blocks of nt threads) that can be resident at once
-int batch_max_groups(int nt, int cs);
+int batch_max_groups(int nt, int cs, const BatchParams& prm);
 void launch_batch_step(int nt, int cs, int ngroups, const BProb* probs, const BDyn* dyn,
                        const int* order, int nprob, int* queue, const BatchParams& prm,
                        const double* rho, double* T, double* E, const double* Ebc, double* wsd,

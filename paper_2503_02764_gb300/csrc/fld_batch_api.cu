@@ -242,7 +242,7 @@ fld_status fld_step_batched(fld_batch* b, const fld_consts* k, const fld_opacity
     prm.fp64 = b->o.precision == FLD_PREC_MIXED_DF ? 0 : 1;
     const int nt = block_threads(b->o);
     const int cl = cluster_size(b, nt);
-    const int maxg = batch_max_groups(nt, cl);
+    const int maxg = batch_max_groups(nt, cl, prm);
     if (maxg < 1) return FLD_ERR_ARG;          // this block/cluster shape cannot be resident
     const int ngroups = std::min(b->nprob, maxg);
     cudaStream_t s = (cudaStream_t)stream;

@@ -9,6 +9,12 @@
 // cluster barrier (or __syncthreads), reductions go through distributed shared memory
 // in a fixed order, and no block ever spins on memory written by another: the launch
 // cannot deadlock and its results do not depend on which group solves which problem.
+//
+// The V-cycles of 2D problems run tile by tile in shared memory (tile2d.cuh): the sweeps, the
+// restriction and the prolongation of one side of a level are one pass over its arrays (32 B
+// a cell and V-cycle in place of about 80) and one barrier in place of three to four. The
+// phases are functions of their own (not inlined): in one function the 512-thread kernel
+// spilled 760 bytes a thread into every loop.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -16,6 +22,7 @@
 #include "df64.cuh"
 #include "fld_batch.cuh"
 #include "fld_device.cuh"
+#include "tile2d.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -100,7 +107,7 @@ __device__ void grp_half(const Grp<CS>& g, const Lvl& L, int color, float* x, fl
 }
 
 template <int CS>
-__device__ void grp_smooth(const Grp<CS>& g, const Lvl& L, int sweeps, float* x, float* t,
+__device__ __noinline__ void grp_smooth(const Grp<CS>& g, const Lvl& L, int sweeps, float* x, float* t,
                            const float* b, const float* K) {
     bool odd = false;
     for (int d = 0; d < L.ndim; ++d) odd |= (L.bclo[d] == FLD_BC_PERIODIC) && (L.n[d] & 1);
@@ -130,7 +137,7 @@ __device__ __forceinline__ void children(const Lvl& F, const Lvl& C, int I, int 
 }
 
 template <int CS>
-__device__ void grp_restrict_K(const Grp<CS>& g, const Lvl& F, const Lvl& C, float scale,
+__device__ __noinline__ void grp_restrict_K(const Grp<CS>& g, const Lvl& F, const Lvl& C, float scale,
                                const float* Kf, float* Kc) {
     for (int P = g.tid; P < (int)C.ncell; P += g.nthr) {
         int c0, c1, c2;
@@ -151,7 +158,7 @@ __device__ void grp_restrict_K(const Grp<CS>& g, const Lvl& F, const Lvl& C, flo
 }
 
 template <int CS>
-__device__ void grp_resid_restrict(const Grp<CS>& g, const Lvl& F, const Lvl& C, const float* x,
+__device__ __noinline__ void grp_resid_restrict(const Grp<CS>& g, const Lvl& F, const Lvl& C, const float* x,
                                    const float* b, const float* K, float* bc, float* xc) {
     for (int P = g.tid; P < (int)C.ncell; P += g.nthr) {
         int c0, c1, c2;
@@ -176,7 +183,7 @@ __device__ void grp_resid_restrict(const Grp<CS>& g, const Lvl& F, const Lvl& C,
 }
 
 template <int CS>
-__device__ void grp_prolong(const Grp<CS>& g, const Lvl& F, const Lvl& C, float* xf,
+__device__ __noinline__ void grp_prolong(const Grp<CS>& g, const Lvl& F, const Lvl& C, float* xf,
                             const float* xc) {
     for (int p = g.tid; p < (int)F.ncell; p += g.nthr) {
         int i, j, k;
@@ -200,7 +207,7 @@ __device__ void grp_prolong(const Grp<CS>& g, const Lvl& F, const Lvl& C, float*
 // Coarsest level: exact dense FP64 solve by the group's first block when small, else
 // red-black sweeps by the whole group.
 template <int CS>
-__device__ void grp_coarse(const Grp<CS>& g, const Lvl& L, float* x, float* t, const float* b,
+__device__ __noinline__ void grp_coarse(const Grp<CS>& g, const Lvl& L, float* x, float* t, const float* b,
                            const float* K, int sweeps, GroupShared& sh) {
     const int n = (int)L.ncell;
     if (n > BMAX_DENSE) {
@@ -258,6 +265,57 @@ __device__ void grp_coarse(const Grp<CS>& g, const Lvl& L, float* x, float* t, c
     g.sync();
 }
 
+// One side of a 2D level, tiles over the group's blocks.
+template <int NT, int CS>
+__device__ __noinline__ void grp_tiles(const Grp<CS>& g, const Lvl& F, const Lvl& C, T2Args a,
+                                       float* tile) {
+    a.R = NT >= 512 ? 48 : 32;
+    a.H = t2_halo(a.sweeps, a.bc != nullptr);
+    const int tx = T2_W - 2 * a.H, ty = a.R - 2 * a.H;
+    const int ntx = (F.n[0] + tx - 1) / tx, nt = ntx * ((F.n[1] + ty - 1) / ty);
+    for (int t = g.rank; t < nt; t += CS) {
+        t2_tile<NT>(F, C, a, (t % ntx) * tx, (t / ntx) * ty, tile);
+        __syncthreads();
+    }
+    g.sync();
+}
+
+// the V-cycle of a 2D problem on tiles; zero: the level-0 iterate starts from zero (not read)
+template <int NT, int CS>
+__device__ void grp_vcycle_tiles(const Grp<CS>& g, const BProb& P, float* F, bool zero, int nu1,
+                                 int nu2, int csweeps, GroupShared& sh, float* tile) {
+    const int L = P.nlev;
+    auto args = [&](int l) {
+        T2Args a{};
+        float* x = F + P.o32[l];
+        const long long n = P.lv[l].ncell;
+        a.b = x + n;
+        a.K = x + 2 * n;
+        return a;
+    };
+    for (int l = 0; l < L - 1; ++l) {
+        T2Args a = args(l);
+        a.xin = l > 0 || zero ? nullptr : F + P.o32[l];
+        a.xout = F + P.o32[l] + 3 * P.lv[l].ncell;
+        a.bc = F + P.o32[l + 1] + P.lv[l + 1].ncell;
+        a.sweeps = nu1;
+        grp_tiles<NT>(g, P.lv[l], P.lv[l + 1], a, tile);
+    }
+    {
+        float* x = F + P.o32[L - 1];
+        const long long n = P.lv[L - 1].ncell;
+        grp_coarse(g, P.lv[L - 1], x, x + 3 * n, x + n, x + 2 * n, csweeps, sh);
+    }
+    for (int l = L - 2; l >= 0; --l) {
+        T2Args a = args(l);
+        a.xin = F + P.o32[l] + 3 * P.lv[l].ncell;
+        a.xout = F + P.o32[l];
+        a.ec = F + P.o32[l + 1];
+        a.sweeps = nu2;
+        grp_tiles<NT>(g, P.lv[l], P.lv[l + 1], a, tile);
+    }
+}
+
 template <int CS>
 __device__ void grp_vcycle(const Grp<CS>& g, const BProb& P, float* F, int nu1, int nu2,
                            int csweeps, GroupShared& sh) {
@@ -287,7 +345,7 @@ __device__ void grp_vcycle(const Grp<CS>& g, const BProb& P, float* F, int nu1, 
 // double-word products and sums: a few units of 2^-48 of |x| and |K x|), r32 = r rounded
 // to FP32; returns the group's sum of r^2.
 template <int CS>
-__device__ double grp_df_resid(const Grp<CS>& g, const Lvl& L, const DfW& wd, const float* xh,
+__device__ __noinline__ double grp_df_resid(const Grp<CS>& g, const Lvl& L, const DfW& wd, const float* xh,
                                const float* xl, const float* bh, const float* bl, const float* Kh,
                                const float* Kl, float* r32, GroupShared& sh) {
     double a2 = 0.0;
@@ -333,23 +391,80 @@ __device__ double grp_df_resid(const Grp<CS>& g, const Lvl& L, const DfW& wd, co
     return grp_sum(a2, sh, g);
 }
 
-// Level-0 residual in FP64: r = b - A x with the level operator's stencil, r32 = r rounded
-// to FP32; returns the group's sum of r^2.
+// Level-0 residual in FP64, r = b - A x with differences first (three FP64 instructions a face),
+// r32 = r rounded to FP32; returns the group's sum of r^2.
 template <int CS>
-__device__ double grp_resid64(const Grp<CS>& g, const Lvl& L, const double* x, const double* b,
-                              const double* K, float* r32, GroupShared& sh) {
+__device__ __noinline__ double grp_resid64(const Grp<CS>& g, const Lvl& L, const double* x,
+                                           const double* b, const double* K, float* r32,
+                                           double one, GroupShared& sh) {
     double a2 = 0.0;
     for (int p = g.tid; p < (int)L.ncell; p += g.nthr) {
-        int i, j, k;
-        decode(L, p, i, j, k);
-        double sw, acc;
-        stencil<double>(L, K, x, i, j, k, p, sw, acc);
-        const double r = b[p] - fma(1.0 + sw, x[p], -acc);
+        int c[3];
+        decode(L, p, c[0], c[1], c[2]);
+        const double xc = x[p], kc = K[p];
+        double r = fma(xc, -one, b[p]);
+        int stride = 1;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            if (d >= L.ndim) break;
+            const int n = L.n[d];
+            double s = 0.0;
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                const int kind = side ? L.bchi[d] : L.bclo[d];
+                const bool edge = side ? c[d] == n - 1 : c[d] == 0;
+                int q = side ? p + stride : p - stride;
+                if (edge) q = kind == FLD_BC_PERIODIC ? (side ? p - (n - 1) * stride
+                                                              : p + (n - 1) * stride) : -1;
+                if (q >= 0) s = fma(fma(kc, one, K[q]), fma(xc, -one, x[q]), s);
+                else if (kind == FLD_BC_DIRICHLET) s = fma(-4.0 * kc, xc, s);
+            }
+            r = fma(0.5 * L.w[d], s, r);
+            stride *= n;
+        }
         r32[p] = (float)r;
         a2 = fma(r, r, a2);
     }
     g.sync();
     return grp_sum(a2, sh, g);
+}
+
+// The limiter on every cell: D; returns the thread's count of cells that failed.
+template <int CS>
+__device__ __noinline__ double grp_limiter(const Grp<CS>& g, const BProb& P, const BatchParams& prm,
+                                           const Opacity& op, const DfConst& KC, const double* E,
+                                           const double* r, const double* T, const double* eb,
+                                           double* D, double one) {
+    const Lvl& L = P.lv[0];
+    BcOff bo;
+    for (int q = 0; q < 6; ++q) bo.off[q] = P.bc_off[q];
+    const double ih[3] = {1.0 / (12.0 * P.h[0]), 1.0 / (12.0 * P.h[1]), 1.0 / (12.0 * P.h[2])};
+    double bad = 0.0;
+    for (int p = g.tid; p < (int)L.ncell; p += g.nthr) {
+        int i, j, k;
+        decode(L, p, i, j, k);
+        double Dv = 0.0, lm;
+        if (!(!prm.fp64 && limiter_cell_df(L, ih, E, r, T, eb, bo, op, KC, prm.limiter, i, j, k, p,
+                                           Dv, lm)) &&
+            !limiter_cell<false>(L, ih, E, r, T, eb, bo, op, prm.c, prm.limiter, i, j, k, p, Dv, lm,
+                                 nullptr, false, one))
+            bad += 1.0;
+        D[p] = Dv;
+    }
+    return bad;
+}
+
+// The exchange in FP64 on every cell, kappa from (rho, T^n), from the solved x.
+template <int CS>
+__device__ __noinline__ void grp_exchange64(const Grp<CS>& g, int n, const double* r, double* T,
+                                            double* E, const double* x, const Opacity& op,
+                                            double dtc, double a_r, double cv) {
+    for (int p = g.tid; p < n; p += g.nthr) {
+        double t = T[p], e = x[p];
+        exchange_cell<false>(r[p], t, e, op, dtc, a_r, cv);
+        T[p] = t;
+        E[p] = e;
+    }
 }
 
 template <int NT, int CS>
@@ -358,8 +473,9 @@ k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
              const int* __restrict__ order, int nprob, int* __restrict__ queue, BatchParams prm,
              const double* __restrict__ rho, double* __restrict__ T, double* __restrict__ E,
              const double* __restrict__ Ebc, double* __restrict__ wsd, float* __restrict__ wsf,
-             BatchStat* __restrict__ stats, unsigned* __restrict__ err) {
+             BatchStat* __restrict__ stats, unsigned* __restrict__ err, double one) {
     __shared__ GroupShared sh;
+    extern __shared__ float tile[];                   // the V-cycles' tiles (2D problems)
     Grp<CS> g;
     if constexpr (CS == 1) g.rank = 0;
     else g.rank = (int)cg::this_cluster().block_rank();
@@ -397,7 +513,21 @@ k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
         float* K32 = x32 + 2 * n0;
         BcOff bo;
         for (int q = 0; q < 6; ++q) bo.off[q] = P.bc_off[q];
-        const double ih[3] = {1.0 / (12.0 * P.h[0]), 1.0 / (12.0 * P.h[1]), 1.0 / (12.0 * P.h[2])};
+        const bool tiled = L0.ndim == 2 && prm.nu1 <= TILE2D_SWEEPS && prm.nu2 <= TILE2D_SWEEPS;
+        // e = 0, then `inner` V-cycles on A e = r
+        auto correction = [&]() {
+            if (!tiled) {
+                for (int p = g.tid; p < n0; p += g.nthr) x32[p] = 0.f;
+                g.sync();
+            }
+            for (int ic = 0; ic < prm.inner; ++ic) {
+                if (tiled)
+                    grp_vcycle_tiles<NT>(g, P, F, ic == 0, prm.nu1, prm.nu2, prm.coarse_sweeps, sh,
+                                         tile);
+                else
+                    grp_vcycle(g, P, F, prm.nu1, prm.nu2, prm.coarse_sweeps, sh);
+            }
+        };
 
         // per-problem constants as double-FP32 pairs
         DfConst KC;
@@ -408,18 +538,7 @@ k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
             KC = {c2.hi, c2.lo, k2.hi, k2.lo, t2.hi, t2.lo, a2.hi, a2.lo, v2.hi, v2.lo};
         }
         // ---- limiter -> D; count domain errors
-        double bad = 0.0;
-        for (int p = g.tid; p < n0; p += g.nthr) {
-            int i, j, k;
-            decode(L0, p, i, j, k);
-            double Dv = 0.0, lm;
-            if (!(!prm.fp64 && limiter_cell_df(L0, ih, E_, r_, T_, eb, bo, op, KC, prm.limiter, i,
-                                               j, k, p, Dv, lm)) &&
-                !limiter_cell<false>(L0, ih, E_, r_, T_, eb, bo, op, prm.c, prm.limiter, i, j, k,
-                                     p, Dv, lm))
-                bad += 1.0;
-            D[p] = Dv;
-        }
+        const double bad = grp_limiter(g, P, prm, op, KC, E_, r_, T_, eb, D, one);
         g.sync();
         const bool bad_any = grp_sum(bad, sh, g) > 0.0;
 
@@ -465,26 +584,17 @@ k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
                                    F + P.o32[l] + 2 * nf, F + P.o32[l + 1] + 2 * nc);
                 }
                 const double bnorm = sqrt(b2);
-                rel = bnorm > 0.0 ? sqrt(grp_resid64(g, L0, x64, b64, K64, b32, sh)) / bnorm : 0.0;
+                rel = bnorm > 0.0 ? sqrt(grp_resid64(g, L0, x64, b64, K64, b32, one, sh)) / bnorm : 0.0;
                 rel0 = rel;
                 while (rel > prm.tol && cyc < prm.max_cycles && isfinite(rel)) {
-                    for (int p = g.tid; p < n0; p += g.nthr) x32[p] = 0.f;
-                    g.sync();
-                    for (int ic = 0; ic < prm.inner; ++ic)
-                        grp_vcycle(g, P, F, prm.nu1, prm.nu2, prm.coarse_sweeps, sh);
+                    correction();
                     for (int p = g.tid; p < n0; p += g.nthr) x64[p] += (double)x32[p];
                     g.sync();
-                    rel = sqrt(grp_resid64(g, L0, x64, b64, K64, b32, sh)) / bnorm;
+                    rel = sqrt(grp_resid64(g, L0, x64, b64, K64, b32, one, sh)) / bnorm;
                     ++cyc;
                 }
                 // ---- the exchange in FP64 with kappa(rho, T^n)
-                const double dtc = dt * prm.c;
-                for (int p = g.tid; p < n0; p += g.nthr) {
-                    double t = T_[p], e_new = x64[p];
-                    exchange_cell<false>(r_[p], t, e_new, op, dtc, prm.a_r, prm.cv);
-                    T_[p] = t;
-                    E_[p] = e_new;
-                }
+                grp_exchange64(g, n0, r_, T_, E_, x64, op, dt * prm.c, prm.a_r, prm.cv);
             } else {
             int ex = 0;
             frexp(b2 > 0.0 ? sqrt(b2 / n0) : 1.0, &ex);
@@ -521,10 +631,7 @@ k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
                       : 0.0;
             rel0 = rel;
             while (rel > prm.tol && cyc < prm.max_cycles && isfinite(rel)) {
-                for (int p = g.tid; p < n0; p += g.nthr) x32[p] = 0.f;
-                g.sync();
-                for (int ic = 0; ic < prm.inner; ++ic)
-                    grp_vcycle(g, P, F, prm.nu1, prm.nu2, prm.coarse_sweeps, sh);
+                correction();
                 for (int p = g.tid; p < n0; p += g.nthr) {
                     const df v = df_add_f({xh[p], xl[p]}, x32[p]);
                     xh[p] = v.hi;
@@ -562,17 +669,18 @@ k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
 }
 
 template <int NT, int CS>
-void launch_one(int nblocks, const BProb* probs, const BDyn* dyn, const int* order, int nprob,
+void launch_one(int nblocks, size_t smem, const BProb* probs, const BDyn* dyn, const int* order, int nprob,
                 int* queue, const BatchParams& prm, const double* rho, double* T, double* E,
                 const double* Ebc, double* wsd, float* wsf, BatchStat* stats, unsigned* err,
                 cudaStream_t s) {
     if constexpr (CS == 1) {
-        k_batch_step<NT, 1><<<nblocks, NT, 0, s>>>(probs, dyn, order, nprob, queue, prm, rho, T, E,
-                                                   Ebc, wsd, wsf, stats, err);
+        k_batch_step<NT, 1><<<nblocks, NT, smem, s>>>(probs, dyn, order, nprob, queue, prm, rho, T,
+                                                      E, Ebc, wsd, wsf, stats, err, 1.0);
     } else {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(nblocks);
         cfg.blockDim = dim3(NT);
+        cfg.dynamicSmemBytes = smem;
         cfg.stream = s;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -582,15 +690,27 @@ void launch_one(int nblocks, const BProb* probs, const BDyn* dyn, const int* ord
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         cudaLaunchKernelEx(&cfg, k_batch_step<NT, CS>, probs, dyn, order, nprob, queue, prm, rho,
-                           T, E, Ebc, wsd, wsf, stats, err);
+                           T, E, Ebc, wsd, wsf, stats, err, 1.0);
     }
 }
 
+// the tiles' shared memory for these sweep counts (none where no problem uses tiles)
+size_t tile_bytes(int nt, int nu1, int nu2) {
+    if (nu1 > TILE2D_SWEEPS || nu2 > TILE2D_SWEEPS) return 0;
+    return sizeof(float) * t2_floats(nt >= 512 ? 48 : 32, true);
+}
+
 template <int NT, int CS>
-int max_groups() {
+int max_groups(size_t smem) {
+    // the attribute belongs to the device that is current
+    if (cudaFuncSetAttribute(k_batch_step<NT, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)tile_bytes(NT, 0, 0)) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
     if constexpr (CS == 1) {
         int nb = 0, dev = 0, nsm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_step<NT, 1>, NT, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_step<NT, 1>, NT, smem);
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         return nb * nsm;
@@ -598,6 +718,7 @@ int max_groups() {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(CS * 64);
         cfg.blockDim = dim3(NT);
+        cfg.dynamicSmemBytes = smem;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = CS;
@@ -627,9 +748,10 @@ int batch_cluster_supported(int cs) { return cs == 1 || cs == 2 || cs == 4 || cs
         default: CALL(NT_, 1);        \
     }
 
-int batch_max_groups(int nt, int cs) {
+int batch_max_groups(int nt, int cs, const BatchParams& prm) {
     int r = 0;
-#define MG(NT_, CS_) r = max_groups<NT_, CS_>()
+    const size_t smem = tile_bytes(nt, prm.nu1, prm.nu2);
+#define MG(NT_, CS_) r = max_groups<NT_, CS_>(smem)
     if (nt == 256) {
         FLD_BATCH_DISPATCH(256, MG)
     } else if (nt == 1024) {
@@ -645,8 +767,9 @@ void launch_batch_step(int nt, int cs, int ngroups, const BProb* probs, const BD
                        const int* order, int nprob, int* queue, const BatchParams& prm,
                        const double* rho, double* T, double* E, const double* Ebc, double* wsd,
                        float* wsf, BatchStat* stats, unsigned* err, cudaStream_t s) {
+    const size_t smem = tile_bytes(nt, prm.nu1, prm.nu2);
 #define LB(NT_, CS_)                                                                        \
-    launch_one<NT_, CS_>(ngroups * CS_, probs, dyn, order, nprob, queue, prm, rho, T, E, Ebc, \
+    launch_one<NT_, CS_>(ngroups * CS_, smem, probs, dyn, order, nprob, queue, prm, rho, T, E, Ebc, \
                          wsd, wsf, stats, err, s)
     if (nt == 256) {
         FLD_BATCH_DISPATCH(256, LB)
