@@ -173,8 +173,7 @@ struct fld_handle {
     std::vector<void*> allocs;
     Prof prof;
     // CUDA graph of the FP32 V-cycle (handle-owned buffers only), replayed per cycle
-    cudaStream_t gs = nullptr;
-    cudaEvent_t gev_in = nullptr, gev_out = nullptr;
+    cudaStream_t gs = nullptr;        // the capture's stream
     cudaGraphExec_t vgraph = nullptr;
     int vgraph_key[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     long long vgraph_nodes = 0;
@@ -701,18 +700,15 @@ fld_status residual_update(fld_handle* h, const double* x, double* xo, double rs
 
 void graph_free(fld_handle* h) {
     if (h->vgraph) cudaGraphExecDestroy(h->vgraph);
-    if (h->gev_in) cudaEventDestroy(h->gev_in);
-    if (h->gev_out) cudaEventDestroy(h->gev_out);
     if (h->gs) cudaStreamDestroy(h->gs);
     h->vgraph = nullptr;
-    h->gev_in = h->gev_out = nullptr;
     h->gs = nullptr;
 }
 
 // e32 = 0, then `inner` FP32 V-cycles on level 0 (each later one continues from the
 // correction so far: its restriction sees the FP32 residual r32 - A e32). With graphs on (and profiling off) the
-// sequence is captured once per option set on a handle-owned stream and replayed;
-// the caller's stream and that stream are ordered through events.
+// sequence is captured once per option set on a handle-owned stream and replayed on the
+// caller's.
 fld_status vcycle32(fld_handle* h, cudaStream_t s) {
     const long long n0 = h->lv[0].ncell;
     const int inner = h->o.inner > 0 ? h->o.inner : 1;
@@ -724,11 +720,7 @@ fld_status vcycle32(fld_handle* h, cudaStream_t s) {
     }
     const int key[8] = {h->o.nu1, h->o.nu2, h->o.smoother, h->o.block, h->o.coarse_sweeps,
                         inner, h->vdepth, h->vsweeps};
-    if (!h->gs) {
-        FLD_CK(cudaStreamCreateWithFlags(&h->gs, cudaStreamNonBlocking));
-        FLD_CK(cudaEventCreateWithFlags(&h->gev_in, cudaEventDisableTiming));
-        FLD_CK(cudaEventCreateWithFlags(&h->gev_out, cudaEventDisableTiming));
-    }
+    if (!h->gs) FLD_CK(cudaStreamCreateWithFlags(&h->gs, cudaStreamNonBlocking));
     if (!h->vgraph || memcmp(key, h->vgraph_key, sizeof(key)) != 0) {
         if (h->vgraph) cudaGraphExecDestroy(h->vgraph);
         h->vgraph = nullptr;
@@ -749,12 +741,8 @@ fld_status vcycle32(fld_handle* h, cudaStream_t s) {
         }
         memcpy(h->vgraph_key, key, sizeof(key));
     }
-    FLD_CK(cudaEventRecord(h->gev_in, s));
-    FLD_CK(cudaStreamWaitEvent(h->gs, h->gev_in, 0));
-    FLD_CK(cudaGraphLaunch(h->vgraph, h->gs));
+    FLD_CK(cudaGraphLaunch(h->vgraph, s));
     g_launches.fetch_add(h->vgraph_nodes);
-    FLD_CK(cudaEventRecord(h->gev_out, h->gs));
-    FLD_CK(cudaStreamWaitEvent(s, h->gev_out, 0));
     return FLD_OK;
 }
 

@@ -359,6 +359,7 @@ template <bool FINE>
 __global__ void __launch_bounds__(256)
 k_amr_smooth(AmrGeom G, AmrRows Rc, AmrRows Rf, int colour, const double* __restrict__ b,
              double* xc, double* xf) {
+    after_previous();
     const int* n = extents<FINE>(G);
     for (int k = blockIdx.z; k < n[2]; k += gridDim.z)
         for (int j = blockIdx.y * blockDim.y + threadIdx.y; j < n[1]; j += gridDim.y * blockDim.y) {
@@ -379,6 +380,7 @@ __global__ void __launch_bounds__(256)
 k_amr_resid(AmrGeom G, AmrRows Rc, AmrRows Rf, const double* __restrict__ b,
             const double* __restrict__ xc, const double* __restrict__ xf,
             double* __restrict__ r, double* __restrict__ partials, double one) {
+    after_previous();
     __shared__ double sh[32];
     const int* n = extents<FINE>(G);
     const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
@@ -405,6 +407,7 @@ k_amr_resid(AmrGeom G, AmrRows Rc, AmrRows Rf, const double* __restrict__ b,
 
 // covered coarse cells: the mean of their fine cells (of v)
 __global__ void k_amr_average(AmrGeom G, const double* __restrict__ vf, double* vc) {
+    after_previous();
     const int nC = amr_ncoarse_cells(G);
     const int n1 = G.nd > 1 ? 2 : 1, n2 = G.nd > 2 ? 2 : 1;
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < nC; p += gridDim.x * blockDim.x) {
@@ -427,6 +430,7 @@ __global__ void k_amr_average(AmrGeom G, const double* __restrict__ vf, double* 
 // x += e on the composite grid: uncovered coarse cells directly, fine cells from their
 // parent (piecewise constant)
 __global__ void k_amr_correct(AmrGeom G, const double* __restrict__ e, double* xc, double* xf) {
+    after_previous();
     const int nC = amr_ncoarse_cells(G), nF = amr_nfine_cells(G);
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < nC + nF; p += gridDim.x * blockDim.x) {
         if (p < nC) {
@@ -475,8 +479,10 @@ void launch_amr_smooth(const AmrGeom& G, const AmrRows& Rc, const AmrRows& Rf, i
     const dim3 blk = pairs > 16 ? dim3(32, 8) : dim3(16, 16);
     const dim3 grd((pairs + blk.x - 1) / blk.x, std::min<int>((n[1] + blk.y - 1) / blk.y, 65535),
                    std::min(n[2], 65535));
-    if (phase >= 2) k_amr_smooth<true><<<grd, blk, 0, s>>>(G, Rc, Rf, phase & 1, bf, xc, xf);
-    else k_amr_smooth<false><<<grd, blk, 0, s>>>(G, Rc, Rf, phase & 1, bc, xc, xf);
+    if (phase >= 2) launch_chained(true, k_amr_smooth<true>, grd, blk, 0, s, G, Rc, Rf, phase & 1,
+                                   bf, xc, xf);
+    else launch_chained(true, k_amr_smooth<false>, grd, blk, 0, s, G, Rc, Rf, phase & 1, bc, xc,
+                        xf);
 }
 
 // two launches; returns the partial sums written (<= nblocks)
@@ -488,19 +494,22 @@ int launch_amr_resid(const AmrGeom& G, const AmrRows& Rc, const AmrRows& Rf, con
         return (int)std::min<long long>(t, nblocks / 2);
     };
     const int nc = blocks(G.nc), nf = blocks(G.nf);
-    k_amr_resid<false><<<nc, 256, 0, s>>>(G, Rc, Rf, bc, xc, xf, rc, partials, 1.0);
-    k_amr_resid<true><<<nf, 256, 0, s>>>(G, Rc, Rf, bf, xc, xf, rf, partials + nc, 1.0);
+    launch_chained(true, k_amr_resid<false>, nc, 256, 0, s, G, Rc, Rf, bc, xc, xf, rc, partials,
+                   1.0);
+    launch_chained(true, k_amr_resid<true>, nf, 256, 0, s, G, Rc, Rf, bf, xc, xf, rf, partials + nc,
+                   1.0);
     return nc + nf;
 }
 
 void launch_amr_average(const AmrGeom& G, const double* vf, double* vc, cudaStream_t s) {
-    k_amr_average<<<amr_blocks((long long)G.nc[0] * G.nc[1] * G.nc[2]), 256, 0, s>>>(G, vf, vc);
+    launch_chained(true, k_amr_average, amr_blocks((long long)G.nc[0] * G.nc[1] * G.nc[2]), 256, 0,
+                   s, G, vf, vc);
 }
 
 void launch_amr_correct(const AmrGeom& G, const double* e, double* xc, double* xf,
                         cudaStream_t s) {
     const long long n = (long long)G.nc[0] * G.nc[1] * G.nc[2] + (long long)G.nf[0] * G.nf[1] * G.nf[2];
-    k_amr_correct<<<amr_blocks(n), 256, 0, s>>>(G, e, xc, xf);
+    launch_chained(true, k_amr_correct, amr_blocks(n), 256, 0, s, G, e, xc, xf);
 }
 
 }  // namespace fld

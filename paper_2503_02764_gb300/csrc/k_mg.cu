@@ -138,6 +138,7 @@ void launch_restrict_K(const Lvl& F, const Lvl& C, double scale, const T* Kf, T*
 template <typename T>
 __global__ void k_smooth(Lvl L, int color, const T* __restrict__ xin, T* __restrict__ xout,
                          const T* __restrict__ b, const T* __restrict__ K) {
+    after_previous();
     const int nrows = L.n[1] * L.n[2];
     for (int r = blockIdx.x; r < nrows; r += gridDim.x) {
         const int j = r % L.n[1], k = r / L.n[1];
@@ -158,7 +159,8 @@ __global__ void k_smooth(Lvl L, int color, const T* __restrict__ xin, T* __restr
 template <typename T>
 void launch_smooth(const Lvl& L, int color, const T* xin, T* xout, const T* b, const T* K,
                    int block, cudaStream_t s) {
-    k_smooth<T><<<rows_grid(L), block, 0, s>>>(L, color, xin, xout, b, K);
+    launch_chained(sizeof(T) == 8 || L.ncell <= CHAIN_CELLS, k_smooth<T>, rows_grid(L), block, 0, s,
+                   L, color, xin, xout, b, K);
 }
 
 // In-place red-black half sweep: only cells of `color` are updated, from neighbours
@@ -212,6 +214,7 @@ __device__ __forceinline__ void rb_cell(const Lvl& L, int i, int j, int k, T* __
 template <typename T>
 __global__ void k_rb_half(Lvl L, int color, T* __restrict__ x, const T* __restrict__ b,
                           const T* __restrict__ K) {
+    after_previous();
     // block = (pairs along x) x (rows along y): neighbouring rows of a tile share L1
     const int ip = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -236,13 +239,15 @@ void launch_rb_half(const Lvl& L, int color, T* x, const T* b, const T* K, cudaS
     const int by = pairs >= 32 ? 8 : 1;
     dim3 block(pairs >= 32 ? bx : (pairs >= 128 ? 128 : ((pairs + 31) / 32) * 32), by);
     dim3 grid((pairs + block.x - 1) / block.x, (L.n[1] + by - 1) / by, L.n[2]);
-    k_rb_half<T><<<grid, block, 0, s>>>(L, color, x, b, K);
+    launch_chained(sizeof(T) == 8 || L.ncell <= CHAIN_CELLS, k_rb_half<T>, grid, block, 0, s, L,
+                   color, x, b, K);
 }
 
 // Coarse right-hand side = average of the fine residuals b - A x over the children.
 template <typename T>
 __global__ void k_resid_restrict(Lvl F, Lvl C, const T* __restrict__ x, const T* __restrict__ b,
                                  const T* __restrict__ K, T* __restrict__ bc) {
+    after_previous();
     for (long long P = blockIdx.x * (long long)blockDim.x + threadIdx.x; P < C.ncell;
          P += (long long)gridDim.x * blockDim.x) {
         int c[3];
@@ -278,11 +283,13 @@ void launch_resid_restrict(const Lvl& F, const Lvl& C, const T* x, const T* b, c
     if constexpr (sizeof(T) == 4)
         if (transfer3_ok(F, C) && !F.fm)
             return launch_resid_restrict3<T>(F, C, x, b, K, bc, red_only, s);
-    k_resid_restrict<T><<<grid_for(C.ncell, block), block, 0, s>>>(F, C, x, b, K, bc);
+    launch_chained(sizeof(T) == 8 || F.ncell <= CHAIN_CELLS, k_resid_restrict<T>, grid_for(C.ncell,
+                   block), block, 0, s, F, C, x, b, K, bc);
 }
 
 template <typename T>
 __global__ void k_prolong(Lvl F, Lvl C, T* __restrict__ xf, const T* __restrict__ xc) {
+    after_previous();
     const int nrows = F.n[1] * F.n[2];
     for (int r = blockIdx.x; r < nrows; r += gridDim.x) {
         const int j = r % F.n[1], k = r / F.n[1];
@@ -310,7 +317,8 @@ __global__ void k_prolong(Lvl F, Lvl C, T* __restrict__ xf, const T* __restrict_
 template <typename T>
 void launch_prolong(const Lvl& F, const Lvl& C, T* xf, const T* xc, int block, cudaStream_t s) {
     if (transfer3_ok(F, C) && !F.pk) return launch_prolong3<T>(F, C, xf, xc, s);
-    k_prolong<T><<<rows_grid(F), block, 0, s>>>(F, C, xf, xc);
+    launch_chained(sizeof(T) == 8 || F.ncell <= CHAIN_CELLS, k_prolong<T>, rows_grid(F), block, 0,
+                   s, F, C, xf, xc);
 }
 
 // Coarsest level: `sweeps` red-black sweeps from x = 0 by one block, in FP64 whatever
@@ -320,6 +328,7 @@ constexpr int MAX_COARSE = 1024;
 template <typename T>
 __global__ void k_coarse_solve(Lvl L, T* __restrict__ x, const T* __restrict__ b,
                                const T* __restrict__ K, int sweeps) {
+    after_previous();
     __shared__ double xs[MAX_COARSE], bs[MAX_COARSE], Ks[MAX_COARSE], nx[MAX_COARSE];
     const int n = (int)L.ncell;
     for (int p = threadIdx.x; p < n; p += blockDim.x) {
@@ -359,6 +368,7 @@ constexpr int MAX_DENSE = 64;
 template <typename T>
 __global__ void k_coarse_dense(Lvl L, T* __restrict__ x, const T* __restrict__ b,
                                const T* __restrict__ K) {
+    after_previous();
     __shared__ double A[MAX_DENSE][MAX_DENSE + 1];
     const int n = (int)L.ncell;
     const int r = threadIdx.x;
@@ -411,9 +421,9 @@ __global__ void k_coarse_dense(Lvl L, T* __restrict__ x, const T* __restrict__ b
 template <typename T>
 void launch_coarse_solve(const Lvl& L, T* x, const T* b, const T* K, int sweeps, cudaStream_t s) {
     if (L.ncell <= MAX_DENSE)
-        k_coarse_dense<T><<<1, MAX_DENSE, 0, s>>>(L, x, b, K);
+        launch_chained(true, k_coarse_dense<T>, 1, MAX_DENSE, 0, s, L, x, b, K);
     else
-        k_coarse_solve<T><<<1, 256, 0, s>>>(L, x, b, K, sweeps);
+        launch_chained(true, k_coarse_solve<T>, 1, 256, 0, s, L, x, b, K, sweeps);
 }
 
 // ----------------------------------------------------------------- FP64 residual + norms
@@ -483,23 +493,25 @@ void launch_resid64(const Lvl& L, const double* x, const double* b, const double
 }
 
 __global__ void k_add_correction(long long n, double* __restrict__ x, const float* __restrict__ e) {
+    after_previous();
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
          p += (long long)gridDim.x * blockDim.x)
         x[p] += (double)e[p];
 }
 
 void launch_add_correction(long long n, double* x, const float* e, cudaStream_t s) {
-    k_add_correction<<<grid_for(n, 256), 256, 0, s>>>(n, x, e);
+    launch_chained(true, k_add_correction, grid_for(n, 256), 256, 0, s, n, x, e);
 }
 
 __global__ void k_to_f32(long long n, const double* __restrict__ v, float* __restrict__ f) {
+    after_previous();
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
          p += (long long)gridDim.x * blockDim.x)
         f[p] = (float)v[p];
 }
 
 void launch_to_f32(long long n, const double* v, float* f, cudaStream_t s) {
-    k_to_f32<<<grid_for(n, 256), 256, 0, s>>>(n, v, f);
+    launch_chained(true, k_to_f32, grid_for(n, 256), 256, 0, s, n, v, f);
 }
 
 __global__ void k_sumsq(long long n, const double* __restrict__ v, double* __restrict__ partials) {
@@ -517,6 +529,7 @@ void launch_sumsq(long long n, const double* v, double* partials, int nblocks, c
 }
 
 __global__ void k_finish_sum(const double* __restrict__ partials, int nparts, double* out) {
+    after_previous();
     __shared__ double sh[32];
     double a = 0.0;
     for (int q = threadIdx.x; q < nparts; q += blockDim.x) a += partials[q];
@@ -525,7 +538,7 @@ __global__ void k_finish_sum(const double* __restrict__ partials, int nparts, do
 }
 
 void launch_finish_sum(const double* partials, int nparts, double* out, cudaStream_t s) {
-    k_finish_sum<<<1, 1024, 0, s>>>(partials, nparts, out);
+    launch_chained(true, k_finish_sum, 1, 1024, 0, s, partials, nparts, out);
 }
 
 // partial sums of the energy density per cell, c_v rho T + E (E alone when rho is null)

@@ -95,6 +95,7 @@ template <int ND, bool OOP>
 __global__ void __launch_bounds__(256)
 k_half64(Lvl L, int color, const double* xin, double* xout, const double* __restrict__ b,
          Coef64 W) {
+    after_previous();
     const int ip = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     const int k = blockIdx.z;
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(256)
 k_norm64(Lvl L, const double* __restrict__ x, const double* __restrict__ b,
          const double* __restrict__ K, Coef64 W, double* __restrict__ partials, int tx, int ty,
          double one) {
+    after_previous();
     __shared__ double sh[32];
     double a2 = 0.0;
     const int ntx = (L.n[0] + tx - 1) / tx, nty = (L.n[1] + ty - 1) / ty;
@@ -167,6 +169,7 @@ template <int ND, bool RED>
 __global__ void __launch_bounds__(128)
 k_restrict64(Lvl F, Lvl C, const double* __restrict__ x, const double* __restrict__ b,
              const double* __restrict__ K, Coef64 W, double* __restrict__ bc, double one) {
+    after_previous();
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
     const int J = blockIdx.y * blockDim.y + threadIdx.y;
     const int Kc = blockIdx.z;
@@ -229,11 +232,13 @@ void launch_half64(const Lvl& L, int color, const double* xin, double* xout, con
     const int pairs = (L.n[0] + 1) / 2;
     const dim3 blk = rows_block(pairs), grd = rows_grid64(L, pairs, blk);
     if (xin == xout) {
-        if (L.ndim == 3) k_half64<3, false><<<grd, blk, 0, s>>>(L, color, xin, xout, b, W);
-        else k_half64<2, false><<<grd, blk, 0, s>>>(L, color, xin, xout, b, W);
+        if (L.ndim == 3) launch_chained(true, k_half64<3, false>, grd, blk, 0, s, L, color, xin,
+                                        xout, b, W);
+        else launch_chained(true, k_half64<2, false>, grd, blk, 0, s, L, color, xin, xout, b, W);
     } else {
-        if (L.ndim == 3) k_half64<3, true><<<grd, blk, 0, s>>>(L, color, xin, xout, b, W);
-        else k_half64<2, true><<<grd, blk, 0, s>>>(L, color, xin, xout, b, W);
+        if (L.ndim == 3) launch_chained(true, k_half64<3, true>, grd, blk, 0, s, L, color, xin,
+                                        xout, b, W);
+        else launch_chained(true, k_half64<2, true>, grd, blk, 0, s, L, color, xin, xout, b, W);
     }
 }
 
@@ -242,8 +247,9 @@ int launch_norm64(const Lvl& L, const double* x, const double* b, const double* 
     const int tx = L.n[0] > 16 ? 32 : 16, ty = 256 / tx;
     const long long tiles = (long long)((L.n[0] + tx - 1) / tx) * ((L.n[1] + ty - 1) / ty) * L.n[2];
     const int nb = (int)std::min<long long>(tiles, nblocks);
-    if (L.ndim == 3) k_norm64<3><<<nb, 256, 0, s>>>(L, x, b, K, W, partials, tx, ty, 1.0);
-    else k_norm64<2><<<nb, 256, 0, s>>>(L, x, b, K, W, partials, tx, ty, 1.0);
+    if (L.ndim == 3) launch_chained(true, k_norm64<3>, nb, 256, 0, s, L, x, b, K, W, partials, tx,
+                                    ty, 1.0);
+    else launch_chained(true, k_norm64<2>, nb, 256, 0, s, L, x, b, K, W, partials, tx, ty, 1.0);
     return nb;
 }
 
@@ -254,11 +260,11 @@ void launch_restrict64(const Lvl& F, const Lvl& C, const double* x, const double
     const dim3 grd((C.n[0] + blk.x - 1) / blk.x, (C.n[1] + blk.y - 1) / blk.y, C.n[2]);
     if (F.ndim == 3) {
         if (red_only && transfer3_ok(F, C))
-            k_restrict64<3, true><<<grd, blk, 0, s>>>(F, C, x, b, K, W, bc, 1.0);
+            launch_chained(true, k_restrict64<3, true>, grd, blk, 0, s, F, C, x, b, K, W, bc, 1.0);
         else
-            k_restrict64<3, false><<<grd, blk, 0, s>>>(F, C, x, b, K, W, bc, 1.0);
+            launch_chained(true, k_restrict64<3, false>, grd, blk, 0, s, F, C, x, b, K, W, bc, 1.0);
     } else {
-        k_restrict64<2, false><<<grd, blk, 0, s>>>(F, C, x, b, K, W, bc, 1.0);
+        launch_chained(true, k_restrict64<2, false>, grd, blk, 0, s, F, C, x, b, K, W, bc, 1.0);
     }
 }
 

@@ -119,6 +119,7 @@ template <int TX, int TY, int MINB>
 __global__ void __launch_bounds__(ZmShape<TX, TY>::NT, MINB)
 k_rb_zmarch(Lvl L, const float* __restrict__ xin, float* __restrict__ xout,
             const float* __restrict__ b, const float* __restrict__ K, int cz) {
+    after_previous();
     using SH = ZmShape<TX, TY>;
     constexpr int PL = SH::PL, XW = SH::XW, CPR = SH::CPR;
     extern __shared__ __align__(16) float zsm[];
@@ -372,8 +373,8 @@ void launch_rb_sweep(const Lvl& L, const T* xin, T* xout, const T* b, const T* K
         const int cz = zm_chunk(L);
         const int tiles = ((L.n[0] + ZM_TX - 1) / ZM_TX) * ((L.n[1] + ZM_TY - 1) / ZM_TY);
         const int nch = (L.n[2] + cz - 1) / cz;
-        k_rb_zmarch<ZM_TX, ZM_TY, ZM_MINB>
-            <<<tiles * nch, ZmMain::NT, ZmMain::SMEM, s>>>(L, xin, xout, b, K, cz);
+        launch_chained(L.ncell <= CHAIN_CELLS, k_rb_zmarch<ZM_TX, ZM_TY, ZM_MINB>, tiles * nch,
+                       ZmMain::NT, ZmMain::SMEM, s, L, xin, xout, b, K, cz);
     }
 }
 

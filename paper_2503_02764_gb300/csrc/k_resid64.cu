@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(RZ_NT, 5)
 k_resid64z(Lvl L, const double* __restrict__ x, const float* __restrict__ e,
            double* __restrict__ xo, const double* __restrict__ b, const double* __restrict__ K,
            float* __restrict__ r32, double* __restrict__ partials, int cz, double one) {
+    after_previous();
     __shared__ double XS[(RZ_TY + 2) * RZ_PW], KS[(RZ_TY + 2) * RZ_PW];
     __shared__ double FX[RZ_TY * (RZ_TX + 1)], FY[(RZ_TY + 1) * RZ_TX];
     __shared__ double sh[32];
@@ -246,6 +247,7 @@ __global__ void __launch_bounds__(RZ_NT)
 k_resid64_2d(Lvl L, const double* __restrict__ x, const float* __restrict__ e,
              double* __restrict__ xo, const double* __restrict__ b, const double* __restrict__ K,
              float* __restrict__ r32, double* __restrict__ partials, double one) {
+    after_previous();
     __shared__ double XS[(RZ_TY + 2) * RZ_PW], KS[(RZ_TY + 2) * RZ_PW];
     __shared__ double FX[RZ_TY * (RZ_TX + 1)], FY[(RZ_TY + 1) * RZ_TX];
     __shared__ double sh[32];
@@ -321,7 +323,7 @@ int launch_resid64_2d(const Lvl& L, const double* x, const float* e, double* xo,
     const long long tiles = (long long)((L.n[0] + RZ_TX - 1) / RZ_TX) *
                             ((L.n[1] + RZ_TY - 1) / RZ_TY);
     const int nb = (int)std::min<long long>(tiles, nblocks);
-    k_resid64_2d<<<nb, RZ_NT, 0, s>>>(L, x, e, xo, b, K, r32, partials, 1.0);
+    launch_chained(true, k_resid64_2d, nb, RZ_NT, 0, s, L, x, e, xo, b, K, r32, partials, 1.0);
     return nb;
 }
 
@@ -354,7 +356,8 @@ int launch_resid64z(const Lvl& L, const double* x, const float* e, double* xo, c
     }
     const int cz = (L.n[2] + best - 1) / best;
     const int nch = (L.n[2] + cz - 1) / cz;
-    k_resid64z<<<tiles * nch, RZ_NT, 0, s>>>(L, x, e, xo, b, K, r32, partials, cz, 1.0);
+    launch_chained(L.ncell <= CHAIN_CELLS, k_resid64z, tiles * nch, RZ_NT, 0, s, L, x, e, xo, b, K,
+                   r32, partials, cz, 1.0);
     return tiles * nch;
 }
 

@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(UZ_NT, 5)
 k_resid_update(Lvl L, const double* __restrict__ x, const float* __restrict__ e,
                double* __restrict__ xo, const float* __restrict__ K, float* __restrict__ r32,
                double* __restrict__ partials, int cz, float rs, float bs, double one) {
+    after_previous();
     __shared__ float ES[(UZ_TY + 2) * UZ_PW], KS[(UZ_TY + 2) * UZ_PW];
     __shared__ double sh[32];
 
@@ -250,6 +251,7 @@ k_resid_update(Lvl L, const double* __restrict__ x, const float* __restrict__ e,
 // the first two groups, out[2] the largest of the third.
 __global__ void k_finish_update(const double* __restrict__ partials, int nparts, double* out0,
                                 double* out1, double* out2) {
+    after_previous();
     __shared__ double sh[32];
     double a = 0.0, b = 0.0;
     float m = 0.f;
@@ -289,14 +291,14 @@ int launch_resid_update(const Lvl& L, const double* x, const float* e, double* x
     int nch = std::max(1, std::min(nblocks / tiles, (L.n[2] + 15) / 16));
     const int cz = (L.n[2] + nch - 1) / nch;
     nch = (L.n[2] + cz - 1) / cz;
-    k_resid_update<<<tiles * nch, UZ_NT, 0, s>>>(L, x, e, xo, K, r32, partials, cz, rs, bs,
-                                                  1.0);
+    launch_chained(L.ncell <= CHAIN_CELLS, k_resid_update, tiles * nch, UZ_NT, 0, s, L, x, e, xo, K,
+                   r32, partials, cz, rs, bs, 1.0);
     return tiles * nch;
 }
 
 void launch_finish_update(const double* partials, int nparts, double* out0, double* out1,
                           double* out2, cudaStream_t s) {
-    k_finish_update<<<1, 1024, 0, s>>>(partials, nparts, out0, out1, out2);
+    launch_chained(true, k_finish_update, 1, 1024, 0, s, partials, nparts, out0, out1, out2);
 }
 
 }  // namespace fld

@@ -164,6 +164,7 @@ __device__ void tail_dense(const Lvl& L, T* __restrict__ x, const T* __restrict_
 // FM: the levels' face mean (0 arithmetic, 1 harmonic), fixed per instantiation
 template <typename T, int FM>
 __global__ void __launch_bounds__(TAIL_THREADS) k_vcycle_tail(TailLevels<T> t) {
+    after_previous();
     __shared__ double A[TAIL_MAX_DENSE][TAIL_MAX_DENSE + 1];
     extern __shared__ __align__(16) unsigned char tail_smem[];
     T* xs[TAIL_MAX_LEVELS];
@@ -218,9 +219,9 @@ template <typename T>
 void launch_vcycle_tail(const TailLevels<T>& t, cudaStream_t s) {
     const size_t sm = tail_smem_bytes<T>(t.L, t.n);
     if (t.L[0].fm)
-        k_vcycle_tail<T, 1><<<1, TAIL_THREADS, sm, s>>>(t);
+        launch_chained(true, k_vcycle_tail<T, 1>, 1, TAIL_THREADS, sm, s, t);
     else
-        k_vcycle_tail<T, 0><<<1, TAIL_THREADS, sm, s>>>(t);
+        launch_chained(true, k_vcycle_tail<T, 0>, 1, TAIL_THREADS, sm, s, t);
 }
 
 // Opt the tail kernels into TAIL_SMEM_MAX bytes of dynamic shared memory, once per device

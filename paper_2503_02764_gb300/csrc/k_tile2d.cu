@@ -15,6 +15,7 @@ namespace {
 constexpr int T2_NT = 512;
 
 __global__ void __launch_bounds__(T2_NT) k_tile2d(Lvl F, Lvl C, T2Args a) {
+    after_previous();
     extern __shared__ float t2[];
     t2_tile<T2_NT>(F, C, a, blockIdx.x * (T2_W - 2 * a.H), blockIdx.y * (a.R - 2 * a.H), t2);
 }
@@ -47,7 +48,8 @@ void launch_tile2d(const Lvl& F, const Lvl& C, const float* xin, float* xout, co
     a.R = big ? 48 : 32;
     const int ty = a.R - 2 * a.H;
     const dim3 grid((F.n[0] + tx - 1) / tx, (F.n[1] + ty - 1) / ty);
-    k_tile2d<<<grid, T2_NT, sizeof(float) * t2_floats(a.R, t2_odd(F)), s>>>(F, C, a);
+    launch_chained(true, k_tile2d, grid, T2_NT, sizeof(float) * t2_floats(a.R, t2_odd(F)), s, F, C,
+                   a);
 }
 
 }  // namespace fld

@@ -77,6 +77,7 @@ bool transfer3_ok(const Lvl& F, const Lvl& C) {
 template <typename T>
 __global__ void k_resid_restrict3(Lvl F, Lvl C, const T* __restrict__ x, const T* __restrict__ b,
                                   const T* __restrict__ K, T* __restrict__ bc) {
+    after_previous();
     const int I = blockIdx.x * 32 + threadIdx.x;
     const int J = blockIdx.y * blockDim.y + threadIdx.y;
     const int Kc = blockIdx.z;
@@ -182,6 +183,7 @@ __global__ void k_resid_restrict3(Lvl F, Lvl C, const T* __restrict__ x, const T
 template <typename T>
 __global__ void k_restrict_red3(Lvl F, Lvl C, const T* __restrict__ x, const T* __restrict__ b,
                                 const T* __restrict__ K, T* __restrict__ bc) {
+    after_previous();
     const int I = blockIdx.x * 32 + threadIdx.x;
     const int J = blockIdx.y * blockDim.y + threadIdx.y;
     const int Kc = blockIdx.z;
@@ -284,6 +286,7 @@ __global__ void k_restrict_red3(Lvl F, Lvl C, const T* __restrict__ x, const T* 
 
 template <typename T>
 __global__ void k_prolong3(Lvl F, Lvl C, T* __restrict__ xf, const T* __restrict__ xc) {
+    after_previous();
     const int I = blockIdx.x * 32 + threadIdx.x;
     const int J = blockIdx.y * blockDim.y + threadIdx.y;
     const int Kc = blockIdx.z;
@@ -373,16 +376,19 @@ void launch_resid_restrict3(const Lvl& F, const Lvl& C, const T* x, const T* b, 
     dim3 block(32, 4);
     dim3 grid((C.n[0] + 31) / 32, (C.n[1] + 3) / 4, C.n[2]);
     if (red_only)
-        k_restrict_red3<T><<<grid, block, 0, s>>>(F, C, x, b, K, bc);
+        launch_chained(sizeof(T) == 8 || F.ncell <= CHAIN_CELLS, k_restrict_red3<T>, grid, block, 0,
+                       s, F, C, x, b, K, bc);
     else
-        k_resid_restrict3<T><<<grid, block, 0, s>>>(F, C, x, b, K, bc);
+        launch_chained(sizeof(T) == 8 || F.ncell <= CHAIN_CELLS, k_resid_restrict3<T>, grid, block,
+                       0, s, F, C, x, b, K, bc);
 }
 
 template <typename T>
 void launch_prolong3(const Lvl& F, const Lvl& C, T* xf, const T* xc, cudaStream_t s) {
     dim3 block(32, 4);
     dim3 grid((C.n[0] + 31) / 32, (C.n[1] + 3) / 4, C.n[2]);
-    k_prolong3<T><<<grid, block, 0, s>>>(F, C, xf, xc);
+    launch_chained(sizeof(T) == 8 || F.ncell <= CHAIN_CELLS, k_prolong3<T>, grid, block, 0, s, F, C,
+                   xf, xc);
 }
 
 template void launch_resid_restrict3<float>(const Lvl&, const Lvl&, const float*, const float*,
