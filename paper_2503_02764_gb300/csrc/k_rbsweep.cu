@@ -260,31 +260,74 @@ k_rb_zmarch(Lvl L, const float* __restrict__ xin, float* __restrict__ xout,
     int pp1 = slot_of(z0), pp2 = slot_of(z0 + 1), pp3 = slot_of(z0 + 2);
     static_assert(ZM_D == 2 && ZM_R == 7, "the rotation below holds planes k-3 .. k+3");
     const bool ring_warp = (tid & ~31) < 2 * nrow + 2 * ncol;   // warp-uniform
-    float* xo = xout + (long long)gy0 * nx + gx;
 
     // ---- the march. Step k: planes <= k + 1 have landed; red(k) on the tile and its ring
     // (in place in the shared copy) and black(k - 2), which reads planes k - 3 .. k - 1
     // only. Both are evaluated unconditionally (so their arithmetic interleaves) and only
     // the stores are predicated. The copy of plane k + 3 goes into the slot of plane k - 4,
     // last read by black(k - 3) in the previous step.
+    //
+    // The sweep is bound by the issue of shared-memory instructions (27 reads a step with
+    // every value read where it is used), so a thread keeps K and x of its own two rows over
+    // planes k - 3 .. k + 1 in registers: row A is the one whose cell is red in the first step,
+    // row B the other, and they change roles every step. A step reads the two rows' new
+    // plane, the x neighbours, the outer y neighbours and b: 18 reads.
     issue(z0 - 2, pm1);
     issue(z0 - 1, p00);
     issue(z0, pp1);
     issue(z0 + 1, pp2);
-    for (int k = z0 - 1; k <= z1 + 1; ++k) {
+    const int q0 = (gx + gy0 + z0 - 1) & 1;
+    const int cA = c0 + q0 * XW, cB = c0 + (1 - q0) * XW;
+    const int yA = q0 ? XW : -XW;                // the outer neighbour of row A; B's is -yA
+    float kA[5], kB[5], xA[5], xB[5];            // planes k - 3 .. k + 1
+    zm_wait<ZM_D>();
+    __syncthreads();
+    kA[2] = zsm[pm1 + cA + PL];
+    kB[2] = zsm[pm1 + cB + PL];
+    xA[2] = zsm[pm1 + cA];
+    xB[2] = zsm[pm1 + cB];
+    kA[3] = zsm[p00 + cA + PL];
+    kB[3] = zsm[p00 + cB + PL];
+    xA[3] = zsm[p00 + cA];
+    xB[3] = zsm[p00 + cB];
+    kA[0] = kA[1] = kB[0] = kB[1] = xA[0] = xA[1] = xB[0] = xB[1] = 0.f;
+    // one step with red row R (offset cr, outer neighbour at yr) and black row S
+    auto step = [&](int k, float (&kR)[5], float (&xR)[5], float (&kS)[5], float (&xS)[5], int cr,
+                    int cb, int yr, bool ar, bool ab, float* outr, float* outb) {
         zm_wait<ZM_D - 1>();
         __syncthreads();
         issue(k + 3, pp3);
         const bool do_red = k <= z1 && zm_axis(k, nz, zper) >= 0;
         const bool do_black = k - 2 >= z0;
-        // red(k): the red row of the pair (parity of gz = parity of k: periodic extents
-        // are even, ghost planes are not updated)
-        const int q = (gx + gy0 + k) & 1;
-        const int cr = c0 + q * XW, cb = cr + (1 - 2 * q) * XW;
-        const float vr = zm_relax<XW, PL>(zsm, p00 + cr, pm1 + cr, pp1 + cr, hx, hy, hz);
-        // black(k - 2): the other row of the pair at plane k - 2 (same parity as k)
-        const float vb = zm_relax<XW, PL>(zsm, pm2 + cb, pm3 + cb, pm1 + cb, hx, hy, hz);
-        const float vrb = zsm[pm2 + cr];             // its red cell, updated two steps ago
+        kR[4] = zsm[pp1 + cr + PL];
+        xR[4] = zsm[pp1 + cr];
+        kS[4] = zsm[pp1 + cb + PL];
+        xS[4] = zsm[pp1 + cb];
+        // the cell of row r at plane index m (1: k - 2, 3: k) in slot o; t the other row
+        auto relax = [&](const float (&kr)[5], const float (&xr)[5], const float (&kt)[5],
+                         const float (&xt)[5], int m, int o, int yo) {
+            const float kc = kr[m];
+            float f = (kc + zsm[o + PL - 1]) * hx;
+            float sw = f, acc = f * zsm[o - 1];
+            f = (kc + zsm[o + PL + 1]) * hx;
+            sw += f;
+            acc = fmaf(f, zsm[o + 1], acc);
+            f = (kc + zsm[o + PL + yo]) * hy;
+            sw += f;
+            acc = fmaf(f, zsm[o + yo], acc);
+            f = (kc + kt[m]) * hy;
+            sw += f;
+            acc = fmaf(f, xt[m], acc);
+            f = (kc + kr[m - 1]) * hz;
+            sw += f;
+            acc = fmaf(f, xr[m - 1], acc);
+            f = (kc + kr[m + 1]) * hz;
+            sw += f;
+            acc = fmaf(f, xr[m + 1], acc);
+            return __fdividef(zsm[o + 2 * PL] + acc, 1.0f + sw);
+        };
+        const float vr = relax(kR, xR, kS, xS, 3, p00 + cr, yr);
+        const float vb = relax(kS, xS, kR, xR, 1, pm2 + cb, -yr);
         if (ring_warp) {
             const bool rsel = (rpar + k) & 1;
             const int cg = rsel ? rc1 : rc0;
@@ -292,16 +335,40 @@ k_rb_zmarch(Lvl L, const float* __restrict__ xin, float* __restrict__ xout,
             const float vg = zm_relax<XW, PL>(zsm, p00 + cq, pm1 + cq, pp1 + cq, hx, hy, hz);
             if (do_red && cg >= 0) zsm[p00 + cg] = vg;
         }
-        if (do_red && (q ? act1 : act0)) zsm[p00 + cr] = vr;
+        if (do_red && ar) {
+            zsm[p00 + cr] = vr;
+            xR[3] = vr;
+        }
         if (do_black) {
-            // the pair's plane k - 2 (its row span checked in the debug build)
-            float* o = xo + (long long)(k - 2) * plane;
-            if (act0) o = xout + fld_span(o - xout, act1 ? nx + 1 : 1, L.ncell);
-            if (act0) o[0] = q ? vb : vrb;
-            if (act1) o[nx] = q ? vrb : vb;
+            // the pair's plane k - 2: row S's cell relaxed now, row R's two steps ago
+            if (ar) outr[0] = xR[1];
+            if (ab) outb[0] = vb;
         }
         const int t = pm3;
         pm3 = pm2; pm2 = pm1; pm1 = p00; p00 = pp1; pp1 = pp2; pp2 = pp3; pp3 = t;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            kR[e] = kR[e + 1];
+            xR[e] = xR[e + 1];
+            kS[e] = kS[e + 1];
+            xS[e] = xS[e + 1];
+        }
+    };
+    const bool actA = q0 ? act1 : act0, actB = q0 ? act0 : act1;
+    // the rows' cells of plane k - 2 in xout, checked in the debug build where they are written
+    long long oA = (long long)(z0 - 3) * plane + (long long)(gy0 + q0) * nx + gx;
+    long long oB = (long long)(z0 - 3) * plane + (long long)(gy0 + 1 - q0) * nx + gx;
+    auto at = [&](long long o, int k, bool act) {
+        return xout + (act && k - 2 >= z0 ? fld_at(o, L.ncell) : 0);
+    };
+    for (int k = z0 - 1; k <= z1 + 1; ++k) {
+        step(k, kA, xA, kB, xB, cA, cB, yA, actA, actB, at(oA, k, actA), at(oB, k, actB));
+        oA += plane;
+        oB += plane;
+        if (++k > z1 + 1) break;
+        step(k, kB, xB, kA, xA, cB, cA, -yA, actB, actA, at(oB, k, actB), at(oA, k, actA));
+        oA += plane;
+        oB += plane;
     }
     zm_wait<0>();
 }
