@@ -5,6 +5,7 @@
 #include "df64.cuh"
 #include "fix64.cuh"
 #include "fld_internal.cuh"
+#include "logtab.cuh"
 
 namespace fld {
 
@@ -292,6 +293,68 @@ __device__ __forceinline__ double exchange_root(double alpha, double beta, doubl
         if (fabs(dx) <= 4e-16 * x) break;
     }
     return x;
+}
+
+// Fractional coordinate of v on a uniform axis of n nodes, clamped to [0, n - 1] by integer
+// comparisons (a NaN goes to the first node): the node below (at most n - 2) and the fraction
+// above it.
+__device__ __forceinline__ int table_node(double v, double v0, double inv, int n,
+                                          double& f) {
+    double x = (v - v0) * inv;
+    const long long b = __double_as_longlong(x), top = __double_as_longlong(f64_of_count(n - 1));
+    if (b < 0 || b > 0x7FF0000000000000LL) x = 0.0;
+    else if (b > top) x = __longlong_as_double(top);
+    const unsigned hi = (unsigned)__double2hiint(x);
+    const int e = (int)(hi >> 20) - 1023;
+    // floor: the integer bits of the significand (x < 2^31)
+    const unsigned m = __funnelshift_l((unsigned)__double2loint(x), (hi & 0xFFFFFu) | 0x100000u, 11);
+    const int i = min(e < 0 ? 0 : (int)(m >> (31 - e)), n - 2);
+    f = x - f64_of_count(i);
+    return i;
+}
+
+// kappa0 10^(bilinear interpolant of the log10 kappa table) at (log10 rho, log10 T), the
+// coordinates clamped to the table, so every read stays inside the nr x nt array (nr, nt >= 2 on
+// the host). Out of line, with scalar arguments, so the kernels' register allocation for the
+// other laws is what it is without tables. 43 FP64 instructions (about 95 with the CUDA library's
+// log10 and exp10, FP64 clamps and conversions): a limiter with tables on 160 x 144 x 128 takes
+// LIMUS us, 706 before.
+static __device__ __noinline__ double opacity_table(const double* __restrict__ tab, int nr,
+                                                    int nt, double lr0, double ilr, double lt0,
+                                                    double ilt, double kappa0, double rho,
+                                                    double T) {
+    double fx, fy;
+    const int i = table_node(tab_log10(rho), lr0, ilr, nr, fx);
+    const int j = table_node(tab_log10(T), lt0, ilt, nt, fy);
+    const double* t = tab + (long long)j * nr + i;
+    const double lo = fma(fx, t[1] - t[0], t[0]);
+    const double hi = fma(fx, t[nr + 1] - t[nr], t[nr]);
+    return kappa0 * tab_exp10(fma(fy, hi - lo, lo));
+}
+
+// kTables = false compiles the table law out (callers that never receive it)
+template <bool kTables = true>
+__device__ __forceinline__ double opacity_eval(const Opacity& op, double rho, double T) {
+    if (op.kind == FLD_OPACITY_CONST) return op.kappa0;
+    if (kTables && op.kind == FLD_OPACITY_TABLE)
+        return opacity_table(op.tab, op.nr, op.nt, op.lr0, op.ilr, op.lt0, op.ilt, op.kappa0,
+                             rho, T);
+    const double fr = (op.a_rho == 1.0) ? rho : pow(rho, op.a_rho);
+    double ft;
+    if (op.a_T == 0.0) {
+        ft = 1.0;
+    } else if (op.a_T == -3.5) {            // Kramers-like law: T^-3.5 = (T^-1/2)^7
+        if (in_f32_range(T)) {
+            const double y = rsqrt_nr(T, 2);
+            const double y2 = y * y;
+            ft = y2 * y2 * y2 * y;
+        } else {
+            ft = 1.0 / (T * T * T * sqrt(T));
+        }
+    } else {
+        ft = pow(T, op.a_T);
+    }
+    return op.kappa0 * fr * ft;
 }
 
 // kappa rho of a cell with positive finite rho and T; false if kappa is not positive and finite.
