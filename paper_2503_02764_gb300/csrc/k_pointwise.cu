@@ -265,9 +265,15 @@ k_coupling(Lvl L, double3 inv12h, const double* __restrict__ E,
 
 // blocks of 32 x 8 cells, or of a line's cells in a row
 static dim3 cell_block(const Lvl& L) { return L.n[1] > 1 ? dim3(32, 8) : dim3(256, 1); }
+// and a thread's planes: up to four, as long as six blocks an SM remain (the launch constants are
+// loaded once a thread; the double-FP32 limiter of 256^3 takes 801 us with one plane a thread)
 static dim3 cell_grid(const Lvl& L, dim3 blk) {
-    return dim3((L.n[0] + blk.x - 1) / blk.x, std::min<int>((L.n[1] + blk.y - 1) / blk.y, 65535),
-                std::min(L.n[2], 65535));
+    const int gx = (L.n[0] + blk.x - 1) / blk.x;
+    const int gy = std::min<int>((L.n[1] + blk.y - 1) / blk.y, 65535);
+    int gz = std::min(L.n[2], 65535);
+    while (gz > 1 && 4LL * gz > L.n[2] && (long long)gx * gy * (gz / 2) >= 6LL * num_sms())
+        gz = (gz + 1) / 2;
+    return dim3(gx, gy, gz);
 }
 
 void launch_coupling(const Lvl& L, const double* h, const double* E, const double* rho,
