@@ -48,10 +48,9 @@ __device__ __forceinline__ double f64_of(float f) {
     return (double)f;
 }
 
-// a + b and a - b as FMAs whose multiplier `one` (1.0) arrives at run time, so the compiler
-// cannot turn them back into adds: the result is the same rounded sum, and on this GPU an
-// FP64 add holds the FP64 pipe about twice as long as an FMA (measured: per-cell FP64 add,
-// multiply and FMA counts against the pipe's busy time in three kernels).
+// a + b and a - b as FMAs whose multiplier `one` (1.0) arrives at run time: the same rounded
+// sum at the same cost (FP64 adds, multiplications and FMAs hold the pipe alike: 19.2 SM cycles
+// a warp, each measured in a loop of its own).
 __device__ __forceinline__ double addf(double a, double b, double one) { return fma(a, one, b); }
 __device__ __forceinline__ double subf(double a, double b, double one) { return fma(b, -one, a); }
 
@@ -82,6 +81,11 @@ __device__ __forceinline__ float f32_of_i(double v) {
     return __uint_as_float(r | sg);
 }
 
+// ISO: the three axis weights are equal. A face then keeps its sum and its difference instead of
+// their product, each cell adds both its faces of an axis to one sum by FMAs, and the weight
+// enters once: 16 FP64 instructions a cell in place of 19 (256^3: 829 us, 977 us with the fluxes,
+// which unequal weights keep).
+template <bool ISO>
 __global__ void __launch_bounds__(RZ_NT, 5)
 k_resid64z(Lvl L, const double* __restrict__ x, const float* __restrict__ e,
            double* __restrict__ xo, const double* __restrict__ b, const double* __restrict__ K,
@@ -89,6 +93,7 @@ k_resid64z(Lvl L, const double* __restrict__ x, const float* __restrict__ e,
     after_previous();
     __shared__ double XS[(RZ_TY + 2) * RZ_PW], KS[(RZ_TY + 2) * RZ_PW];
     __shared__ double FX[RZ_TY * (RZ_TX + 1)], FY[(RZ_TY + 1) * RZ_TX];
+    __shared__ double DX[ISO ? RZ_TY * (RZ_TX + 1) : 1], DY[ISO ? (RZ_TY + 1) * RZ_TX : 1];
     __shared__ double sh[32];
 
     const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
@@ -179,7 +184,7 @@ k_resid64z(Lvl L, const double* __restrict__ x, const float* __restrict__ e,
     };
 
     double acc2 = 0.0;
-    double xprev = 0.0, kprev = 0.0, gzprev = 0.0, part = 0.0;
+    double xprev = 0.0, kprev = 0.0, gzprev = 0.0, part = 0.0, accz = 0.0;
     Raw cur = {}, nxt = {};
     load_raw(z0, cur);
     if (act) {
@@ -209,9 +214,27 @@ k_resid64z(Lvl L, const double* __restrict__ x, const float* __restrict__ e,
         auto flux = [&](double kc, double kq, double xc, double xq) {
             return addf(kc, kq, one) * subf(xc, xq, one);
         };
-        double gz = 0.0;
-        if (act) gz = flux(kk, kprev, xk, xprev);
-        if (inplane && act) {
+        double gz = 0.0, dz = 0.0;                 // ISO: the face's sum and difference
+        if (act) {
+            if (ISO) {
+                gz = addf(kk, kprev, one);
+                dz = subf(xk, xprev, one);
+            } else {
+                gz = flux(kk, kprev, xk, xprev);
+            }
+        }
+        if (ISO && inplane && act) {
+            auto face = [&](double* f, double* d, int c, int q) {
+                *f = addf(KS[c], KS[q], one);
+                *d = subf(XS[c], XS[q], one);
+            };
+            const int fx = ly * (RZ_TX + 1) + lx, fy = ly * RZ_TX + lx;
+            face(FX + fx, DX + fx, so, so - 1);
+            if (lx == ax - 1) face(FX + fx + 1, DX + fx + 1, so + 1, so);
+            face(FY + fy, DY + fy, so, so - RZ_PW);
+            if (ly == ay - 1) face(FY + fy + RZ_TX, DY + fy + RZ_TX, so + RZ_PW, so);
+        }
+        if (!ISO && inplane && act) {
             FX[ly * (RZ_TX + 1) + lx] = flux(KS[so], KS[so - 1], XS[so], XS[so - 1]);
             if (lx == ax - 1)
                 FX[ly * (RZ_TX + 1) + lx + 1] = flux(KS[so + 1], KS[so], XS[so + 1], XS[so]);
@@ -221,15 +244,26 @@ k_resid64z(Lvl L, const double* __restrict__ x, const float* __restrict__ e,
         }
         // the plane below is complete: its +z face is this plane's -z face
         if (act && k - 1 >= z0) {
-            const double r = fma(-hz, subf(gzprev, gz, one), part);
+            // ISO: part is b - x, accz the sum so far (its x, y and lower z faces)
+            const double r = ISO ? fma(hz, fma(gz, dz, accz), part)
+                                 : fma(-hz, subf(gzprev, gz, one), part);
             if (r32) r32[fld_at((long long)(k - 1) * plane + own, L.ncell)] = f32_of(r);
             acc2 = fma(r, r, acc2);
         }
         __syncthreads();
         if (inplane && act) {
             const int fx = ly * (RZ_TX + 1) + lx, fy = ly * RZ_TX + lx;
-            const double r = fma(-hx, subf(FX[fx], FX[fx + 1], one), subf(cur.b, xk, one));
-            part = fma(-hy, subf(FY[fy], FY[fy + RZ_TX], one), r);
+            if (ISO) {
+                double acc = -gz * dz;
+                acc = fma(FX[fx], -DX[fx], acc);
+                acc = fma(FX[fx + 1], DX[fx + 1], acc);
+                acc = fma(FY[fy], -DY[fy], acc);
+                accz = fma(FY[fy + RZ_TX], DY[fy + RZ_TX], acc);
+                part = subf(cur.b, xk, one);
+            } else {
+                const double r = fma(-hx, subf(FX[fx], FX[fx + 1], one), subf(cur.b, xk, one));
+                part = fma(-hy, subf(FY[fy], FY[fy + RZ_TX], one), r);
+            }
         }
         xprev = xk;
         kprev = kk;
@@ -336,7 +370,7 @@ int launch_resid64z(const Lvl& L, const double* x, const float* e, double* xo, c
     int slots = (dev >= 0 && dev < 64) ? g_rz_slots[dev] : 0;
     if (slots <= 0) {
         int occ = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_resid64z, RZ_NT, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_resid64z<true>, RZ_NT, 0);
         slots = std::max(1, num_sms() * occ);
         if (dev >= 0 && dev < 64) g_rz_slots[dev] = slots;
     }
@@ -356,8 +390,9 @@ int launch_resid64z(const Lvl& L, const double* x, const float* e, double* xo, c
     }
     const int cz = (L.n[2] + best - 1) / best;
     const int nch = (L.n[2] + cz - 1) / cz;
-    launch_chained(L.ncell <= CHAIN_CELLS, k_resid64z, tiles * nch, RZ_NT, 0, s, L, x, e, xo, b, K,
-                   r32, partials, cz, 1.0);
+    const bool iso = L.w[0] == L.w[1] && L.w[0] == L.w[2];
+    launch_chained(L.ncell <= CHAIN_CELLS, iso ? k_resid64z<true> : k_resid64z<false>, tiles * nch,
+                   RZ_NT, 0, s, L, x, e, xo, b, K, r32, partials, cz, 1.0);
     return tiles * nch;
 }
 
