@@ -581,7 +581,6 @@ void vcycle(fld_handle* h, LevelBufs<T>* P, int l, bool zero, cudaStream_t s) {
         run(h, f32 ? "tail32" : "tail64", l, L.ncell, s, [&] { launch_vcycle_tail<T>(t, s); });
         return;
     }
-    const int bs = blk(h);
     // fused sweeps swap the buffers, so an even number of them brings the iterate back
     // to B.x; with an odd nu1 + nu2 the last sweep of the cycle runs in place
     const int nu1 = h->o.nu1, nu2 = h->o.nu2;
@@ -601,12 +600,12 @@ void vcycle(fld_handle* h, LevelBufs<T>* P, int l, bool zero, cudaStream_t s) {
                 return launch_restrict64(L, C, cur, B.b, B.K, h->w64[l], P[l + 1].b,
                                          nu1 > 0 && !L.fm, s);
         }
-        launch_resid_restrict<T>(L, C, cur, B.b, B.K, P[l + 1].b, bs, nu1 > 0, s);
+        launch_resid_restrict<T>(L, C, cur, B.b, B.K, P[l + 1].b, nu1 > 0, s);
     });
     zero_level<T>(h, P, l + 1, s);
     vcycle<T>(h, P, l + 1, true, s);
     run(h, f32 ? "prolong32" : "prolong64", l, L.ncell, s,
-        [&] { launch_prolong<T>(L, C, cur, P[l + 1].x, bs, s); });
+        [&] { launch_prolong<T>(L, C, cur, P[l + 1].x, s); });
     smooth<T>(h, B, l, nu2, f2, cur, oth, s);
 }
 

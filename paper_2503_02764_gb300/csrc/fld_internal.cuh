@@ -291,9 +291,9 @@ template <typename T>
 void launch_prolong3(const Lvl& F, const Lvl& C, T* xf, const T* xc, cudaStream_t s);
 template <typename T>
 void launch_resid_restrict(const Lvl& F, const Lvl& C, const T* x, const T* b, const T* K,
-                           T* bc, int block, bool red_only, cudaStream_t s);
+                           T* bc, bool red_only, cudaStream_t s);
 template <typename T>
-void launch_prolong(const Lvl& F, const Lvl& C, T* xf, const T* xc, int block, cudaStream_t s);
+void launch_prolong(const Lvl& F, const Lvl& C, T* xf, const T* xc, cudaStream_t s);
 template <typename T>
 void launch_coarse_solve(const Lvl& L, T* x, const T* b, const T* K, int sweeps, cudaStream_t s);
 void launch_resid64(const Lvl& L, const double* x, const double* b, const double* K,
