@@ -140,12 +140,14 @@ typedef struct {
     int coarse_sweeps;  /* red-black sweeps of the coarsest-level solve             */
     int limiter;        /* FLD_LIMITER_LP, _DIFFUSION (lambda = 1/3) or _MINERBO    */
     int block;          /* threads per block of the row-mapped kernels (0 = default) */
-    int smoother;       /* 0: in-place red and black half sweeps (levels with no odd
-                           periodic extent; others as 1); 1: two out-of-place half
-                           sweeps; 2: one z-marching pass per sweep (3D FP32 levels
-                           with nx a multiple of 4, nx >= 16, even periodic extents;
-                           others as 0). The levels from 8^3 cells down run in one
-                           single-block launch whatever the smoother.                  */
+    int smoother;       /* how the red-black sweeps run; the updates are the same. 0, 2: the
+                           fastest form of the level: one z-marching pass per sweep (3D
+                           FP32 levels with nx a multiple of 4, nx >= 16, even periodic
+                           extents), one pass per side of the V-cycle on tiles (2D FP32
+                           levels with at most 4 sweeps a side), in-place half sweeps
+                           (other levels with no odd periodic extent), else as 1; 1: two
+                           out-of-place half sweeps. The levels from 8^3 cells down run in
+                           one single-block launch whatever the smoother.              */
     int graph;          /* single grid: replay the FP32 V-cycle from a CUDA graph
                            captured on first use; batched step: capture the step on
                            the first call with given field pointers and replay it       */
@@ -154,7 +156,8 @@ typedef struct {
     int inner;          /* MIXED/MIXED_DF: FP32 V-cycles per refinement step (the later
                            ones continue from the previous correction); 0 means 1      */
     int direct1d;       /* 1D grids: 1 solves the tridiagonal system directly (parallel
-                           cyclic reduction in FP64, a dozen launches; stats report one
+                           cyclic reduction in FP64; one launch for the whole substep or
+                           solve up to 8192 cells, a dozen above; stats report one
                            cycle), 0 runs V-cycles as in 2D and 3D                      */
     int diag;           /* diagnostics filled into fld_stats by fld_diffuse and fld_step
                            when a stats pointer is given: FLD_DIAG_ENERGY adds the total

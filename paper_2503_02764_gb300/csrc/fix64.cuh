@@ -1,6 +1,6 @@
 // FP64 results with few FP64 instructions.
 //
-// An FP64 instruction holds this GPU's FP64 pipe for 16 cycles of an SM, in which its four
+// An FP64 instruction of a warp holds this GPU's FP64 pipe for 16 to 19 cycles of an SM, in which its four
 // schedulers can issue 64 other instructions. The routines here do the bulk of an operation in
 // FP32 and integer arithmetic and leave to FP64 only what fixes the last bits:
 //   fix_div, fix_sqrt   a double-FP32 approximation (~2^-39) from an FP32 reciprocal (square
@@ -31,8 +31,8 @@ __device__ __forceinline__ f32pair split_pos(double v) {
 }
 
 // h + l as FP64 (h positive and normal, |l| below 64 units of h), l rounded to 2^-15 units of h:
-// 2^-39 of the value, which the residual correction takes to 2^-61. (An F2I conversion would
-// hold the FP64 pipe like two FP64 instructions: 1.5 * 2^23 rounds to an integer instead.)
+// 2^-39 of the value, which the residual correction takes to 2^-61 (1.5 * 2^23 rounds to the
+// integer).
 __device__ __forceinline__ double join_pos(float h, float l) {
     const unsigned u = __float_as_uint(h);
     const float per = __uint_as_float((277u << 23) - (u & 0x7F800000u));   // 1 / unit of h

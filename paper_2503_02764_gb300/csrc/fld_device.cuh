@@ -318,7 +318,7 @@ __device__ __forceinline__ int table_node(double v, double v0, double inv, int n
 // the host). Out of line, with scalar arguments, so the kernels' register allocation for the
 // other laws is what it is without tables. 43 FP64 instructions (about 95 with the CUDA library's
 // log10 and exp10, FP64 clamps and conversions): a limiter with tables on 160 x 144 x 128 takes
-// LIMUS us, 706 before.
+// 378 us, 706 before.
 static __device__ __noinline__ double opacity_table(const double* __restrict__ tab, int nr,
                                                     int nt, double lr0, double ilr, double lt0,
                                                     double ilt, double kappa0, double rho,
@@ -386,7 +386,7 @@ __device__ __forceinline__ bool kapparho(const Opacity& op, double r, double t, 
 // c E / (a + g + sqrt(a^2 + 2 a g)): one or two square roots and one division, by the routines
 // of fix64.cuh where the operands allow it (FP64 issues at a small fraction of the FP32 rate
 // here: LP with a Kramers opacity took 46 FP64 instructions with the gradient in FP64 and
-// Newton-Raphson roots, and takes 23). Operands outside the FP32 range take R itself. kr_out
+// Newton-Raphson roots, and takes 26). Operands outside the FP32 range take R itself. kr_out
 // receives kappa rho (the exchange of the same substep reuses it). Returns false on a domain
 // error.
 //
@@ -482,7 +482,7 @@ __device__ __forceinline__ void exchange_cell_kr(double r, double kr, double& t,
                                                  double dtc, double a_r, double cv,
                                                  double one = 1.0) {
     const double chi = dtc * kr;
-    const double d1 = fma(chi, one, 1.0);      // 1 + chi as an FMA (an FP64 add costs two)
+    const double d1 = fma(chi, one, 1.0);
     if (!in_f32_range(d1)) {                   // divided by 1 + chi: nothing overflows
         const double inv1 = 1.0 / d1, w = chi * inv1;
         const double beta = w * a_r, q = fma(w, er, r * cv * t);

@@ -2,7 +2,7 @@
 //
 // FP64 instructions bound these kernels, not memory: this GPU issues 0.6 T of them a second,
 // 64 times fewer than FP32 ones. Evaluating the face coefficients from K in every half
-// sweep took 46 FP64 issue slots per updated cell (six sums, six weightings, the diagonal
+// sweep took about 40 FP64 instructions per updated cell (six sums, six weightings, the diagonal
 // and a division): 651 us per half sweep of a 256^3 level. The coefficients do not change
 // during a solve, so they are formed once per level and solve:
 //   wx, wy, wz  the weight mean(K_p, K_q) w_d of the face towards the lower neighbour along
@@ -57,7 +57,7 @@ k_coef64(Lvl L, double3 half, const double* __restrict__ K, Coef64 W, double one
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
         const double hd = d == 0 ? half.x : d == 1 ? half.y : half.z, dw = L.w[d];
-        // sums of two cells' K as FMAs by a run-time one (an FP64 add takes two issue slots)
+        // the sum of two cells' K
         auto ksum = [&](int q) { return L.fm ? fsum2(kc, K[q], 1) : fma(K[q], one, kc); };
         double w = 0.0;
         if (nb[d].lo >= 0) {

@@ -26,8 +26,7 @@
 // periodic neighbours, or the wall ghosts e = 0 with K = 3 K_wall for Dirichlet and -K_wall
 // for Neumann) sit in shared memory, the planes below and above in registers, the next
 // plane's words are loaded while the current one is computed. Per cell it moves 32 bytes
-// (x 8 + e 4 + K 4 + r 4 read, x 8 + r 4 written) and issues one FP64 instruction (x + e,
-// an FMA with a unit multiplier).
+// (x 8 + e 4 + K 4 + r 4 read, x 8 + r 4 written) and issues one FP64 instruction (x + e).
 #include <algorithm>
 
 #include "fld_device.cuh"
