@@ -44,13 +44,14 @@ BYTES_PER_CELL = {
     "df_setup": 48.0,         # E, b, K read; their FP32 (hi, lo) pairs written
     "df_finish": 16.0,        # x (hi, lo) read; E written
     "sumsq": 8.0,             # b read
-    "resid64": 28.0,          # x, b, K read; r32 written (mixed) / 24 (fp64)
+    "resid64": 28.0,          # x, b, K read; r32 written (mixed) / x, b, weights read (fp64): 40
+    "coef64": 40.0,           # K read; three face weights, inverse diagonal written
     "resid64x": 40.0,         # x, e32, b, K read; x + e, r32 written
     "resid32": 24.0,          # x, b (FP64), K32 read; r32 written (FP32 arithmetic)
     "resid_upd": 32.0,        # x, e32, K32, r32 read; x + e, r32 written (r - A e in FP32)
     "resid_df": 40.0,         # x (hi, lo), e32, b (hi, lo), K (hi, lo) read; x (hi, lo), r32 written
     "rbhalf32": 10.0,         # one colour: the other colour's x and every K read (faces),
-    "rbhalf64": 20.0,         #   this colour's b read and x written
+    "rbhalf64": 28.0,         #   this colour's b read and x written (fp64: stored weights)
     "rbsweep32": 16.0,        # x, K, b read; x written (both colours in one pass)
     "rbsweep64": 32.0,
     "add_correction": 20.0,   # x, e32 read; x written
@@ -75,15 +76,15 @@ def load_peaks():
 # FP64 operations per cell of the FP64-bound level-0 kernels, counted in their source for
 # an interior cell of the 3D workload (add, multiply = 1 flop, FMA = 2; the FP32 seeds and
 # the integer format conversions are not counted): the FP64 limiter with the Kramers
-# opacity (15 for kappa, 23 for the gradient, 29 for D from one square root and one
-# division), the FP64 exchange given kappa rho (FP32 Newton seed, one FP64 Newton step,
-# E'), the FP64 refinement residual with each face flux evaluated once (3D levels), and
-# the same with the correction x + e added in it.
+# opacity (13 FMAs and 12 multiplications by the instruction counters; the 4th-order differences
+# are in fixed point), the FP64 exchange given kappa rho (FP32 Newton seed, one FP64 Newton
+# step, E'), the FP64 refinement residual with each face's sum and difference formed once (3D
+# levels, equal axis weights), and the same with the correction x + e added in it.
 FP64_FLOPS_PER_CELL = {
-    "limiter": 67.0,
-    "exchange": 29.0,
-    "resid64": 21.0,
-    "resid64x": 22.0,
+    "limiter": 38.0,
+    "exchange": 23.0,
+    "resid64": 22.0,
+    "resid64x": 23.0,
 }
 
 
@@ -533,7 +534,7 @@ def profile_steps(hd, consts, op, P, rho, T, E, ebc, steps, torch, peak_hbm, pre
     def bpc(e):
         b = BYTES_PER_CELL.get(e["name"])
         if e["name"] == "resid64" and prec == 0:
-            b = 24.0
+            b = 40.0
         return b
 
     total_ms = sum(e["ms"] for e in prof)
