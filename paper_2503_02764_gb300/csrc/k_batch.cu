@@ -345,9 +345,12 @@ __device__ void grp_vcycle(const Grp<CS>& g, const BProb& P, float* F, int nu1, 
 // double-word products and sums: a few units of 2^-48 of |x| and |K x|), r32 = r rounded
 // to FP32; returns the group's sum of r^2.
 template <int CS>
-__device__ __noinline__ double grp_df_resid(const Grp<CS>& g, const Lvl& L, const DfW& wd, const float* xh,
-                               const float* xl, const float* bh, const float* bl, const float* Kh,
-                               const float* Kl, float* r32, GroupShared& sh) {
+__device__ __noinline__ double grp_df_resid(const Grp<CS>& g, const Lvl& Lg, const DfW& wg,
+                                            const float* xh, const float* xl, const float* bh,
+                                            const float* bl, const float* Kh, const float* Kl,
+                                            float* r32, GroupShared& sh) {
+    const Lvl L = Lg;      // by value: out of line, the stores to r32 could change what Lg names
+    const DfW wd = wg;
     double a2 = 0.0;
     for (int p = g.tid; p < (int)L.ncell; p += g.nthr) {
         int i, j, k;
@@ -358,9 +361,12 @@ __device__ __noinline__ double grp_df_resid(const Grp<CS>& g, const Lvl& L, cons
         const int c[3] = {i, j, k};
         int stride = 1;
         df dw = {0.f, 0.f};
-        for (int d = 0; d < L.ndim; ++d) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            if (d >= L.ndim) break;
             const int nd = L.n[d];
             df ax = {0.f, 0.f};
+#pragma unroll
             for (int side = 0; side < 2; ++side) {
                 const int kind = side ? L.bchi[d] : L.bclo[d];
                 int q = -1;
@@ -394,9 +400,10 @@ __device__ __noinline__ double grp_df_resid(const Grp<CS>& g, const Lvl& L, cons
 // Level-0 residual in FP64, r = b - A x with differences first (three FP64 instructions a face),
 // r32 = r rounded to FP32; returns the group's sum of r^2.
 template <int CS>
-__device__ __noinline__ double grp_resid64(const Grp<CS>& g, const Lvl& L, const double* x,
+__device__ __noinline__ double grp_resid64(const Grp<CS>& g, const Lvl& Lg, const double* x,
                                            const double* b, const double* K, float* r32,
                                            double one, GroupShared& sh) {
+    const Lvl L = Lg;
     double a2 = 0.0;
     for (int p = g.tid; p < (int)L.ncell; p += g.nthr) {
         int c[3];
@@ -429,13 +436,28 @@ __device__ __noinline__ double grp_resid64(const Grp<CS>& g, const Lvl& L, const
     return grp_sum(a2, sh, g);
 }
 
+// The FP64 routines of the cells that the double-FP32 ones decline, out of line: inlined, their
+// FP64 instructions are executed speculatively by every cell.
+__device__ __noinline__ bool limiter_far(const Lvl& L, const double* ih, const double* E,
+                                         const double* rho, const double* T, const double* eb,
+                                         const BcOff& bo, const Opacity& op, double c, int mode,
+                                         int i, int j, int k, int p, double& D) {
+    double lm;
+    return limiter_cell<false>(L, ih, E, rho, T, eb, bo, op, c, mode, i, j, k, p, D, lm, nullptr,
+                               false);
+}
+__device__ __noinline__ void exchange_far(double r, double& t, double& e, const Opacity& op,
+                                          double dtc, double a_r, double cv) {
+    exchange_cell<false>(r, t, e, op, dtc, a_r, cv);
+}
+
 // The limiter on every cell: D; returns the thread's count of cells that failed.
-template <int CS>
+template <bool DF, int CS>
 __device__ __noinline__ double grp_limiter(const Grp<CS>& g, const BProb& P, const BatchParams& prm,
                                            const Opacity& op, const DfConst& KC, const double* E,
                                            const double* r, const double* T, const double* eb,
                                            double* D, double one) {
-    const Lvl& L = P.lv[0];
+    const Lvl L = P.lv[0];
     BcOff bo;
     for (int q = 0; q < 6; ++q) bo.off[q] = P.bc_off[q];
     const double ih[3] = {1.0 / (12.0 * P.h[0]), 1.0 / (12.0 * P.h[1]), 1.0 / (12.0 * P.h[2])};
@@ -444,11 +466,12 @@ __device__ __noinline__ double grp_limiter(const Grp<CS>& g, const BProb& P, con
         int i, j, k;
         decode(L, p, i, j, k);
         double Dv = 0.0, lm;
-        if (!(!prm.fp64 && limiter_cell_df(L, ih, E, r, T, eb, bo, op, KC, prm.limiter, i, j, k, p,
-                                           Dv, lm)) &&
-            !limiter_cell<false>(L, ih, E, r, T, eb, bo, op, prm.c, prm.limiter, i, j, k, p, Dv, lm,
-                                 nullptr, false, one))
-            bad += 1.0;
+        const bool ok =
+            DF ? limiter_cell_df(L, ih, E, r, T, eb, bo, op, KC, prm.limiter, i, j, k, p, Dv, lm) ||
+                     limiter_far(L, ih, E, r, T, eb, bo, op, prm.c, prm.limiter, i, j, k, p, Dv)
+               : limiter_cell<false>(L, ih, E, r, T, eb, bo, op, prm.c, prm.limiter, i, j, k, p, Dv,
+                                     lm, nullptr, false, one);
+        if (!ok) bad += 1.0;
         D[p] = Dv;
     }
     return bad;
@@ -466,6 +489,33 @@ __device__ __noinline__ void grp_exchange64(const Grp<CS>& g, int n, const doubl
         E[p] = e;
     }
 }
+
+// E back from the scaled pairs, then the exchange in double-FP32 with kappa(rho, T^n).
+template <int CS>
+__device__ __noinline__ void grp_exchange_df(const Grp<CS>& g, int n, const double* r, double* T,
+                                             double* E, const float* xh, const float* xl,
+                                             double invS, const Opacity& opg, const DfConst& KCg,
+                                             double dtc, double a_r, double cv) {
+    const Opacity op = opg;
+    const DfConst KC = KCg;
+    for (int p = g.tid; p < n; p += g.nthr) {
+        const double e_sol = ((double)xh[p] + (double)xl[p]) * invS;
+        double t = T[p], e_new = e_sol;
+        if (!exchange_cell_df(r[p], t, e_new, op, KC)) {
+            t = T[p];
+            e_new = e_sol;
+            exchange_far(r[p], t, e_new, op, dtc, a_r, cv);
+        }
+        T[p] = t;
+        E[p] = e_new;
+    }
+}
+
+// Blocks of 1024 threads, one an SM, keep the half sweeps: a tile has too few cells for them, and
+// no other block fills the time of its barriers and loads (512 problems, MIXED_DF: 45.2 ms with
+// tiles, 40.7 with half sweeps; two blocks of 512 an SM gain, MIXED 43.1 -> 34.0).
+template <int NT>
+constexpr bool TILES = NT < 1024;
 
 template <int NT, int CS>
 __global__ void __launch_bounds__(NT)
@@ -513,7 +563,8 @@ k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
         float* K32 = x32 + 2 * n0;
         BcOff bo;
         for (int q = 0; q < 6; ++q) bo.off[q] = P.bc_off[q];
-        const bool tiled = L0.ndim == 2 && prm.nu1 <= TILE2D_SWEEPS && prm.nu2 <= TILE2D_SWEEPS;
+        const bool tiled = TILES<NT> && L0.ndim == 2 && prm.nu1 <= TILE2D_SWEEPS &&
+                           prm.nu2 <= TILE2D_SWEEPS;
         // e = 0, then `inner` V-cycles on A e = r
         auto correction = [&]() {
             if (!tiled) {
@@ -538,7 +589,9 @@ k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
             KC = {c2.hi, c2.lo, k2.hi, k2.lo, t2.hi, t2.lo, a2.hi, a2.lo, v2.hi, v2.lo};
         }
         // ---- limiter -> D; count domain errors
-        const double bad = grp_limiter(g, P, prm, op, KC, E_, r_, T_, eb, D, one);
+        const double bad =
+            prm.fp64 ? grp_limiter<false>(g, P, prm, op, KC, E_, r_, T_, eb, D, one)
+                     : grp_limiter<true>(g, P, prm, op, KC, E_, r_, T_, eb, D, one);
         g.sync();
         const bool bad_any = grp_sum(bad, sh, g) > 0.0;
 
@@ -642,19 +695,7 @@ k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
                 ++cyc;
             }
             // ---- E back from the scaled iterate, then the exchange with kappa(rho, T^n)
-            const double invS = 1.0 / S;
-            const double dtc = dt * prm.c;
-            for (int p = g.tid; p < n0; p += g.nthr) {
-                const double e_sol = ((double)xh[p] + (double)xl[p]) * invS;
-                double t = T_[p], e_new = e_sol;
-                if (!exchange_cell_df(r_[p], t, e_new, op, KC)) {
-                    t = T_[p];
-                    e_new = e_sol;
-                    exchange_cell<false>(r_[p], t, e_new, op, dtc, prm.a_r, prm.cv);
-                }
-                T_[p] = t;
-                E_[p] = e_new;
-            }
+            grp_exchange_df(g, n0, r_, T_, E_, xh, xl, 1.0 / S, op, KC, dt * prm.c, prm.a_r, prm.cv);
             }
         }
         if (g.rank == 0 && threadIdx.x == 0) {
@@ -696,7 +737,7 @@ void launch_one(int nblocks, size_t smem, const BProb* probs, const BDyn* dyn, c
 
 // the tiles' shared memory for these sweep counts (none where no problem uses tiles)
 size_t tile_bytes(int nt, int nu1, int nu2) {
-    if (nu1 > TILE2D_SWEEPS || nu2 > TILE2D_SWEEPS) return 0;
+    if (nt >= 1024 || nu1 > TILE2D_SWEEPS || nu2 > TILE2D_SWEEPS) return 0;
     return sizeof(float) * t2_floats(nt >= 512 ? 48 : 32, true);
 }
 
