@@ -197,7 +197,8 @@ fld_status step_ars3(fld_wave1d* w, double* U, double t, double dt, fld_stats* s
     g.G3 = w->G3;
     g.t_in = t2;
     g.t_out = t + dt;
-    // a failed stage leaves U as it was (elsewhere the failure was read back above)
+    // A failed stage leaves U as it was: the second one fails too where the first has raised the
+    // domain flag. (Stages of longer lines were read back above.)
     if (w->p.radiation && fld_line_wave_ok(w->h)) g.gate = fld_line_failed(w->h, 1);
     rc = advance(w, g, s);
     return rc != FLD_OK ? rc : finish(w, 2, rs, stats, s);

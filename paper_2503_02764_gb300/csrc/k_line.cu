@@ -253,7 +253,11 @@ k_line(LineArgs g, int lg, LineOut* out, unsigned* err) {
             X[q] = er;
         }
         if (csum(fail) > 0.0) {
-            if (rank == 0 && threadIdx.x == 0) out->failed = 1u;
+            // the flag stops the step's next stage, which would read this one's outputs
+            if (rank == 0 && threadIdx.x == 0) {
+                atomicOr(err, ERRBIT_DOMAIN);
+                out->failed = 1u;
+            }
             return;
         }
         const Wave1dDev& P = g.w.P;
