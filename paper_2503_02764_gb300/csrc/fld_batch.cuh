@@ -45,6 +45,14 @@ int batch_threads_supported(int nt);
 int batch_cluster_supported(int cs);
 // groups (clusters of cs blocks of nt threads) that can be resident at once
 int batch_max_groups(int nt, int cs, const BatchParams& prm);
+// the same, and the launch, for one block size (batch_step.cuh)
+template <int NT>
+int batch_groups(int cs, const BatchParams& prm);
+template <int NT>
+void batch_launch(int cs, int ngroups, const BProb* probs, const BDyn* dyn, const int* order,
+                  int nprob, int* queue, const BatchParams& prm, const double* rho, double* T,
+                  double* E, const double* Ebc, double* wsd, float* wsf, BatchStat* stats,
+                  unsigned* err, cudaStream_t s);
 void launch_batch_step(int nt, int cs, int ngroups, const BProb* probs, const BDyn* dyn,
                        const int* order, int nprob, int* queue, const BatchParams& prm,
                        const double* rho, double* T, double* E, const double* Ebc, double* wsd,

@@ -1,6 +1,6 @@
 // A tile of a 2D FP32 multigrid level in shared memory: (prolongation +) n red-black sweeps
 // (+ residual and restriction), out of place. Shared by the single-grid V-cycle (k_tile2d.cu)
-// and the batched step (k_batch.cu).
+// and the batched step (batch_step.cuh).
 //
 // The tile is loaded with a halo of H cells, and every half sweep relaxes a region one cell
 // smaller on each side (the halo's values are recomputed, not exchanged between tiles): H = 2 n,
