@@ -10,15 +10,16 @@
 // in a fixed order, and no block ever spins on memory written by another: the launch
 // cannot deadlock and its results do not depend on which group solves which problem.
 //
-// The V-cycles of 2D problems run tile by tile in shared memory (tile2d.cuh): the sweeps, the
+// The V-cycles of 2D problems that are large enough or shared by a cluster (batch_tiled in
+// fld_batch.cuh) run tile by tile in shared memory (tile2d.cuh): the sweeps, the
 // restriction and the prolongation of one side of a level are one pass over its arrays (32 B
 // a cell and V-cycle in place of about 80) and one barrier in place of three to four.
 //
 // The phases are left to the compiler to inline: as functions of their own each loop re-reads the
 // level's extents and walls through a pointer (512 problems of 32 to 512 cells a side, blocks of
 // 1024 threads, MIXED_DF: 33.8 ms, inlined 31.6; 512 lines: 2.07 ms, inlined 1.76; blocks of 256
-// on 3D problems: 36.0 ms, inlined 29.4). One translation unit per block size (k_batch_256.cu
-// and the like), since a kernel takes ptxas some 20 s.
+// on 3D problems: 36.0 ms, inlined 29.4). One translation unit per block size, with and
+// without tiles (k_batch_256.cu and the like), since a kernel takes ptxas some 20 s.
 #pragma once
 #include <cooperative_groups.h>
 
@@ -274,12 +275,16 @@ __device__ void grp_coarse(const Grp<CS>& g, const Lvl& L, float* x, float* t, c
 template <int NT, int CS>
 __device__ void grp_tiles(const Grp<CS>& g, const Lvl& F, const Lvl& C, T2Args a,
                           float* tile) {
-    a.R = NT >= 512 ? 48 : 32;
     a.H = t2_halo(a.sweeps, a.bc != nullptr);
-    const int tx = T2_W - 2 * a.H, ty = a.R - 2 * a.H;
+    const int most = batch_tile_rows(NT), tx = T2_W - 2 * a.H, ty = most - 2 * a.H;
     const int ntx = (F.n[0] + tx - 1) / tx, nt = ntx * ((F.n[1] + ty - 1) / ty);
     for (int t = g.rank; t < nt; t += CS) {
-        t2_tile<NT>(F, C, a, (t % ntx) * tx, (t / ntx) * ty, tile);
+        const int y0 = (t / ntx) * ty;
+        // the last tiles along y load the rows that are left (an even number: they restrict
+        // pairs), which is all of a coarse level (600 problems of 64^2, two blocks of 512 each:
+        // 4.42 ms with full tiles, 4.00 so)
+        a.R = min(most, ((F.n[1] - y0 + 1) & ~1) + 2 * a.H);
+        t2_tile<NT>(F, C, a, (t % ntx) * tx, y0, tile);
         __syncthreads();
     }
     g.sync();
@@ -515,14 +520,14 @@ __device__ void grp_exchange_df(const Grp<CS>& g, int n, const double* r, double
     }
 }
 
-// Blocks of 1024 threads, one an SM, keep the half sweeps: a tile has too few cells for them, and
-// no other block fills the time of its barriers and loads (512 problems, MIXED_DF: 45.2 ms with
-// tiles, 40.7 with half sweeps; two blocks of 512 an SM gain, MIXED 43.1 -> 34.0).
-template <int NT>
-constexpr bool TILES = NT < 1024;
-
-template <int NT, int CS>
-__global__ void __launch_bounds__(NT)
+// TILED: with the code and the shared memory of the tiles, for batches with a problem that
+// batch_tiled takes; the others keep their L1 and their registers (256 3D problems, blocks of
+// 512: 13.4 ms with a tile's memory reserved, 12.5 without; 512 lines: 2.07 and 1.72 ms).
+// Unclustered blocks of 256 threads run four an SM without tiles (64 registers): a problem of
+// 17^2 to 193^2 cells leaves most of a block waiting (600 of 65^2: 2.79 ms, three an SM 3.37,
+// two 3.30).
+template <int NT, int CS, bool TILED>
+__global__ void __launch_bounds__(NT, NT == 256 ? (CS == 1 && !TILED ? 4 : 2) : 1024 / NT)
 k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
              const int* __restrict__ order, int nprob, int* __restrict__ queue, BatchParams prm,
              const double* __restrict__ rho, double* __restrict__ T, double* __restrict__ E,
@@ -567,8 +572,7 @@ k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
         float* K32 = x32 + 2 * n0;
         BcOff bo;
         for (int q = 0; q < 6; ++q) bo.off[q] = P.bc_off[q];
-        const bool tiled = TILES<NT> && L0.ndim == 2 && prm.nu1 <= TILE2D_SWEEPS &&
-                           prm.nu2 <= TILE2D_SWEEPS;
+        const bool tiled = TILED && batch_tiled(L0, NT, CS, prm.nu1, prm.nu2);
         // e = 0, then `inner` V-cycles on A e = r
         auto correction = [&]() {
             if (!tiled) {
@@ -713,14 +717,15 @@ k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
     }
 }
 
-template <int NT, int CS>
-void launch_one(int nblocks, size_t smem, const BProb* probs, const BDyn* dyn, const int* order, int nprob,
-                int* queue, const BatchParams& prm, const double* rho, double* T, double* E,
+template <int NT, int CS, bool TILED>
+void launch_one(int nblocks, size_t smem, const BProb* probs, const BDyn* dyn, const int* order,
+                int nprob, int* queue, const BatchParams& prm, const double* rho, double* T, double* E,
                 const double* Ebc, double* wsd, float* wsf, BatchStat* stats, unsigned* err,
                 cudaStream_t s) {
     if constexpr (CS == 1) {
-        k_batch_step<NT, 1><<<nblocks, NT, smem, s>>>(probs, dyn, order, nprob, queue, prm, rho, T,
-                                                      E, Ebc, wsd, wsf, stats, err, 1.0);
+        k_batch_step<NT, 1, TILED><<<nblocks, NT, smem, s>>>(probs, dyn, order, nprob, queue, prm,
+                                                             rho, T, E, Ebc, wsd, wsf, stats, err,
+                                                             1.0);
     } else {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(nblocks);
@@ -734,28 +739,28 @@ void launch_one(int nblocks, size_t smem, const BProb* probs, const BDyn* dyn, c
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        cudaLaunchKernelEx(&cfg, k_batch_step<NT, CS>, probs, dyn, order, nprob, queue, prm, rho,
-                           T, E, Ebc, wsd, wsf, stats, err, 1.0);
+        cudaLaunchKernelEx(&cfg, k_batch_step<NT, CS, TILED>, probs, dyn, order, nprob, queue, prm,
+                           rho, T, E, Ebc, wsd, wsf, stats, err, 1.0);
     }
 }
 
-// the tiles' shared memory for these sweep counts (none where no problem uses tiles)
-size_t tile_bytes(int nt, int nu1, int nu2) {
-    if (nt >= 1024 || nu1 > TILE2D_SWEEPS || nu2 > TILE2D_SWEEPS) return 0;
-    return sizeof(float) * t2_floats(nt >= 512 ? 48 : 32, true);
-}
+// the tiles' shared memory
+template <int NT, bool TILED>
+constexpr size_t TILE_BYTES = TILED ? sizeof(float) * t2_floats(batch_tile_rows(NT), true) : 0;
 
-template <int NT, int CS>
-int max_groups(size_t smem) {
+template <int NT, int CS, bool TILED>
+int max_groups() {
+    constexpr size_t smem = TILE_BYTES<NT, TILED>;
+    const auto kernel = k_batch_step<NT, CS, TILED>;
     // the attribute belongs to the device that is current
-    if (cudaFuncSetAttribute(k_batch_step<NT, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tile_bytes(NT, 0, 0)) != cudaSuccess) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+        cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     if constexpr (CS == 1) {
         int nb = 0, dev = 0, nsm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_step<NT, 1>, NT, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, NT, smem);
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         return nb * nsm;
@@ -772,7 +777,7 @@ int max_groups(size_t smem) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int nc = 0;
-        if (cudaOccupancyMaxActiveClusters(&nc, k_batch_step<NT, CS>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&nc, kernel, &cfg) != cudaSuccess) {
             cudaGetLastError();
             return 0;
         }
@@ -791,35 +796,33 @@ int max_groups(size_t smem) {
 
 }  // namespace
 
-template <int NT>
-int batch_groups(int cs, const BatchParams& prm) {
+template <int NT, bool TILED>
+int batch_groups(int cs) {
     int r = 0;
-    const size_t smem = tile_bytes(NT, prm.nu1, prm.nu2);
-#define MG(CS_) r = max_groups<NT, CS_>(smem)
+#define MG(CS_) r = max_groups<NT, CS_, TILED>()
     FLD_BATCH_DISPATCH(MG)
 #undef MG
     return r;
 }
 
-template <int NT>
+template <int NT, bool TILED>
 void batch_launch(int cs, int ngroups, const BProb* probs, const BDyn* dyn, const int* order,
                   int nprob, int* queue, const BatchParams& prm, const double* rho, double* T,
                   double* E, const double* Ebc, double* wsd, float* wsf, BatchStat* stats,
                   unsigned* err, cudaStream_t s) {
-    const size_t smem = tile_bytes(NT, prm.nu1, prm.nu2);
-#define LB(CS_)                                                                              \
-    launch_one<NT, CS_>(ngroups * CS_, smem, probs, dyn, order, nprob, queue, prm, rho, T, E, \
-                        Ebc, wsd, wsf, stats, err, s)
+#define LB(CS_)                                                                                \
+    launch_one<NT, CS_, TILED>(ngroups * CS_, TILE_BYTES<NT, TILED>, probs, dyn, order, nprob, \
+                               queue, prm, rho, T, E, Ebc, wsd, wsf, stats, err, s)
     FLD_BATCH_DISPATCH(LB)
 #undef LB
 }
 
 // the definitions of one block size
-#define FLD_BATCH_DEFINE(NT_)                                                                   \
-    template int batch_groups<NT_>(int, const BatchParams&);                                     \
-    template void batch_launch<NT_>(int, int, const BProb*, const BDyn*, const int*, int, int*,  \
-                                    const BatchParams&, const double*, double*, double*,         \
-                                    const double*, double*, float*, BatchStat*, unsigned*,       \
-                                    cudaStream_t);
+#define FLD_BATCH_DEFINE(NT_, TILED_)                                                         \
+    template int batch_groups<NT_, TILED_>(int);                                              \
+    template void batch_launch<NT_, TILED_>(int, int, const BProb*, const BDyn*, const int*,  \
+                                            int, int*, const BatchParams&, const double*,     \
+                                            double*, double*, const double*, double*, float*, \
+                                            BatchStat*, unsigned*, cudaStream_t);
 
 }  // namespace fld

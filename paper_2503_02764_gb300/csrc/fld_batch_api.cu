@@ -242,6 +242,9 @@ fld_status fld_step_batched(fld_batch* b, const fld_consts* k, const fld_opacity
     prm.fp64 = b->o.precision == FLD_PREC_MIXED_DF ? 0 : 1;
     const int nt = block_threads(b->o);
     const int cl = cluster_size(b, nt);
+    prm.tiles = std::any_of(b->hp.begin(), b->hp.end(), [&](const BProb& P) {
+        return batch_tiled(P.lv[0], nt, cl, prm.nu1, prm.nu2);
+    });
     const int maxg = batch_max_groups(nt, cl, prm);
     if (maxg < 1) return FLD_ERR_ARG;          // this block/cluster shape cannot be resident
     const int ngroups = std::min(b->nprob, maxg);

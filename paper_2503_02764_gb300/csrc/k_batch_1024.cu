@@ -2,5 +2,5 @@
 #include "batch_step.cuh"
 
 namespace fld {
-FLD_BATCH_DEFINE(1024)
+FLD_BATCH_DEFINE(1024, false)
 }  // namespace fld

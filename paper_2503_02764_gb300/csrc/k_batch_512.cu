@@ -1,6 +1,6 @@
-// The batched step with blocks of 512 threads.
+// The batched step with blocks of 512 threads, half sweeps only.
 #include "batch_step.cuh"
 
 namespace fld {
-FLD_BATCH_DEFINE(512)
+FLD_BATCH_DEFINE(512, false)
 }  // namespace fld

@@ -37,7 +37,7 @@ __host__ __device__ __forceinline__ int t2_halo(int sweeps, bool restricts) {
     return 2 * sweeps + (restricts ? 1 : 0);
 }
 // floats of shared memory of a tile: x, K, b, and a second x on odd periodic extents
-__host__ __device__ __forceinline__ int t2_floats(int R, bool odd) {
+__host__ __device__ constexpr int t2_floats(int R, bool odd) {
     return (odd ? 4 : 3) * T2_W * R;
 }
 __host__ __device__ __forceinline__ bool t2_odd(const Lvl& F) {
