@@ -42,9 +42,11 @@ void launch_amr_correct(const AmrGeom& G, const double* e, double* xc, double* x
                         cudaStream_t s);
 
 // The block's multigrid as the coarse correction (fld_api.cu): the operator of D over dt set up
-// once per solve, then `cycles` V-cycles on A e = r from e = 0, without a read-back.
+// once per solve, then `cycles` V-cycles on A e = r from e = 0, without a read-back. `scale`, a
+// power of two, brings r to order one, where the FP32 V-cycles of the mixed modes hold it.
 fld_status fld_correction_setup(fld_handle* h, double dt, const double* D, const double* r,
                                 cudaStream_t s);
-fld_status fld_correction(fld_handle* h, const double* r, double* e, int cycles, cudaStream_t s);
+fld_status fld_correction(fld_handle* h, const double* r, double scale, double* e, int cycles,
+                          cudaStream_t s);
 
 }  // namespace fld

@@ -233,7 +233,10 @@ fld_status fld_amr_diffuse(fld_amr* a, double dt, const double* Dc, const double
         } else {
             if (cyc == 0) rc = fld_correction_setup(a->hc, dt, a->DH, a->rc, s);
             else if (rel > AMR_SLOW * before) vcycles = std::min(2 * vcycles, AMR_MOST);
-            if (rc == FLD_OK) rc = fld_correction(a->hc, a->rc, a->eH, vcycles, s);
+            int ex = 0;                    // the residual's RMS is about 2^ex
+            std::frexp(std::sqrt(r2 / (double)(a->nC + a->nF)), &ex);
+            const double scale = std::ldexp(1.0, -std::max(-1000, std::min(ex, 1000)));
+            if (rc == FLD_OK) rc = fld_correction(a->hc, a->rc, scale, a->eH, vcycles, s);
             if (rc != FLD_OK) return rc;
         }
         launch_amr_correct(G, a->eH, Ec, Ef, s);

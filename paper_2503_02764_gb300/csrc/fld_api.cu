@@ -1433,7 +1433,7 @@ fld_status fld::fld_correction_setup(fld_handle* h, double dt, const double* D, 
     return FLD_OK;
 }
 
-fld_status fld::fld_correction(fld_handle* h, const double* r, double* e, int cycles,
+fld_status fld::fld_correction(fld_handle* h, const double* r, double scale, double* e, int cycles,
                                cudaStream_t s) {
     const long long n = h->ncell;
     if (h->o.precision == FLD_PREC_FP64) {
@@ -1442,14 +1442,14 @@ fld_status fld::fld_correction(fld_handle* h, const double* r, double* e, int cy
         h->d64[0].x = e;
         for (int c = 0; c < cycles; ++c) vcycle<double>(h, h->d64, 0, false, s);
     } else {
-        run(h, "to_f32", 0, n, s, [&] { launch_to_f32(n, r, h->d32[0].b, s); });
+        run(h, "to_f32", 0, n, s, [&] { launch_to_f32(n, r, scale, h->d32[0].b, s); });
         const int inner = h->o.inner;
         h->o.inner = cycles;
         const fld_status rc = vcycle32(h, s);
         h->o.inner = inner;
         if (rc != FLD_OK) return rc;
-        FLD_CK(cudaMemsetAsync(e, 0, sizeof(double) * n, s));
-        run(h, "add_correction", 0, n, s, [&] { launch_add_correction(n, e, h->d32[0].x, s); });
+        run(h, "from_f32", 0, n, s,
+            [&] { launch_from_f32(n, h->d32[0].x, 1.0 / scale, e, s); });
     }
     FLD_CK(cudaGetLastError());
     return FLD_OK;

@@ -298,7 +298,9 @@ template <typename T>
 void launch_coarse_solve(const Lvl& L, T* x, const T* b, const T* K, int sweeps, cudaStream_t s);
 void launch_resid64(const Lvl& L, const double* x, const double* b, const double* K,
                     float* r32, double* partials, int nblocks, int block, cudaStream_t s);
-void launch_to_f32(long long n, const double* v, float* f, cudaStream_t s);
+// f = scale v rounded to FP32, and v = scale f
+void launch_to_f32(long long n, const double* v, double scale, float* f, cudaStream_t s);
+void launch_from_f32(long long n, const float* f, double scale, double* v, cudaStream_t s);
 void launch_add_correction(long long n, double* x, const float* e, cudaStream_t s);
 // direct solve of a 1D level's system by parallel cyclic reduction (k_tridiag.cu), and one
 // step of iterative refinement of x with it; w holds 12 n + 1 doubles; both return the

@@ -8,7 +8,7 @@
 // right-hand sides stay in shared memory, neighbours are read from the blocks that own them
 // (distributed shared memory), and a cluster barrier (~0.3 us) takes the place of each
 // launch. Longer lines keep the launches over the whole GPU (k_tridiag.cu): at 8192 cells the
-// cluster's FP64 issue (13 steps of 17 instructions a row on 8 SMs, ~60 us) costs as much as
+// cluster's FP64 issue (13 steps of 14 instructions a row on 8 SMs, ~60 us) costs as much as
 // their launches do.
 //
 // The system and the method are those of k_tridiag.cu (parallel cyclic reduction,

@@ -519,15 +519,28 @@ void launch_add_correction(long long n, double* x, const float* e, cudaStream_t 
     launch_chained(true, k_add_correction, grid_for(n, 256), 256, 0, s, n, x, e);
 }
 
-__global__ void k_to_f32(long long n, const double* __restrict__ v, float* __restrict__ f) {
+__global__ void k_to_f32(long long n, const double* __restrict__ v, double scale,
+                         float* __restrict__ f) {
     after_previous();
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
          p += (long long)gridDim.x * blockDim.x)
-        f[p] = (float)v[p];
+        f[p] = (float)(scale * v[p]);
 }
 
-void launch_to_f32(long long n, const double* v, float* f, cudaStream_t s) {
-    launch_chained(true, k_to_f32, grid_for(n, 256), 256, 0, s, n, v, f);
+void launch_to_f32(long long n, const double* v, double scale, float* f, cudaStream_t s) {
+    launch_chained(true, k_to_f32, grid_for(n, 256), 256, 0, s, n, v, scale, f);
+}
+
+__global__ void k_from_f32(long long n, const float* __restrict__ f, double scale,
+                           double* __restrict__ v) {
+    after_previous();
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
+         p += (long long)gridDim.x * blockDim.x)
+        v[p] = scale * (double)f[p];
+}
+
+void launch_from_f32(long long n, const float* f, double scale, double* v, cudaStream_t s) {
+    launch_chained(true, k_from_f32, grid_for(n, 256), 256, 0, s, n, f, scale, v);
 }
 
 __global__ void k_sumsq(long long n, const double* __restrict__ v, double* __restrict__ partials) {
