@@ -147,6 +147,17 @@ void debug_attach_all() {
 }
 }  // namespace fld
 
+// A captured FP32 V-cycle sequence and the options it was captured for. A handle keeps as many as a
+// composite solve's doubling counts of V-cycles need (1, 2, 4, 8 and 16), and one more: with a
+// single one a stiff solve captured and instantiated it anew at each doubling (64^3 block, MIXED, a
+// step of 1000 explicit ones: 34.5 ms, 32.6 with the graphs kept).
+struct VGraph {
+    cudaGraphExec_t exec = nullptr;
+    int key[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    long long nodes = 0;
+};
+constexpr int VGRAPHS = 6;
+
 struct fld_handle {
     fld_grid g;
     fld_opts o;
@@ -174,9 +185,8 @@ struct fld_handle {
     Prof prof;
     // CUDA graph of the FP32 V-cycle (handle-owned buffers only), replayed per cycle
     cudaStream_t gs = nullptr;        // the capture's stream
-    cudaGraphExec_t vgraph = nullptr;
-    int vgraph_key[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    long long vgraph_nodes = 0;
+    VGraph vgraphs[VGRAPHS] = {};
+    int vgraph_next = 0;              // the entry that a graph not found replaces
     // first level of the single-launch V-cycle tail (-1: none); set when the levels are built
     int tail_start = -1;
     // levels the V-cycles of the current solve use (the last one solved by vsweeps
@@ -710,16 +720,18 @@ fld_status residual_update(fld_handle* h, const double* x, double* xo, double rs
 }
 
 void graph_free(fld_handle* h) {
-    if (h->vgraph) cudaGraphExecDestroy(h->vgraph);
+    for (VGraph& v : h->vgraphs) {
+        if (v.exec) cudaGraphExecDestroy(v.exec);
+        v = VGraph();
+    }
     if (h->gs) cudaStreamDestroy(h->gs);
-    h->vgraph = nullptr;
     h->gs = nullptr;
 }
 
 // e32 = 0, then `inner` FP32 V-cycles on level 0 (each later one continues from the
-// correction so far: its restriction sees the FP32 residual r32 - A e32). With graphs on (and profiling off) the
-// sequence is captured once per option set on a handle-owned stream and replayed on the
-// caller's.
+// correction so far: its restriction sees the FP32 residual r32 - A e32). With graphs on (and
+// profiling off) the sequence is captured once per option set on a handle-owned stream and
+// replayed on the caller's.
 fld_status vcycle32(fld_handle* h, cudaStream_t s) {
     const long long n0 = h->lv[0].ncell;
     const int inner = h->o.inner > 0 ? h->o.inner : 1;
@@ -732,9 +744,14 @@ fld_status vcycle32(fld_handle* h, cudaStream_t s) {
     const int key[8] = {h->o.nu1, h->o.nu2, h->o.smoother, h->o.block, h->o.coarse_sweeps,
                         inner, h->vdepth, h->vsweeps};
     if (!h->gs) FLD_CK(cudaStreamCreateWithFlags(&h->gs, cudaStreamNonBlocking));
-    if (!h->vgraph || memcmp(key, h->vgraph_key, sizeof(key)) != 0) {
-        if (h->vgraph) cudaGraphExecDestroy(h->vgraph);
-        h->vgraph = nullptr;
+    VGraph* v = nullptr;
+    for (VGraph& q : h->vgraphs)
+        if (q.exec && memcmp(key, q.key, sizeof(key)) == 0) v = &q;
+    if (!v) {
+        v = &h->vgraphs[h->vgraph_next];
+        h->vgraph_next = (h->vgraph_next + 1) % VGRAPHS;
+        if (v->exec) cudaGraphExecDestroy(v->exec);
+        v->exec = nullptr;
         cudaGraph_t g = nullptr;
         const long long before = g_launches.load();
         FLD_CK(cudaStreamBeginCapture(h->gs, cudaStreamCaptureModeThreadLocal));
@@ -742,18 +759,18 @@ fld_status vcycle32(fld_handle* h, cudaStream_t s) {
             cudaMemsetAsync(h->d32[0].x, 0, sizeof(float) * n0, h->gs);
         for (int c = 0; c < inner; ++c) vcycle<float>(h, h->d32, 0, c == 0, h->gs);
         FLD_CK(cudaStreamEndCapture(h->gs, &g));
-        h->vgraph_nodes = g_launches.load() - before;
-        g_launches.fetch_sub(h->vgraph_nodes);       // counted per replay below
-        cudaError_t e = cudaGraphInstantiate(&h->vgraph, g, 0);
+        v->nodes = g_launches.load() - before;
+        g_launches.fetch_sub(v->nodes);       // counted per replay below
+        cudaError_t e = cudaGraphInstantiate(&v->exec, g, 0);
         cudaGraphDestroy(g);
         if (e != cudaSuccess) {
-            h->vgraph = nullptr;
+            v->exec = nullptr;
             return cuda_fail(e);
         }
-        memcpy(h->vgraph_key, key, sizeof(key));
+        memcpy(v->key, key, sizeof(key));
     }
-    FLD_CK(cudaGraphLaunch(h->vgraph, s));
-    g_launches.fetch_add(h->vgraph_nodes);
+    FLD_CK(cudaGraphLaunch(v->exec, s));
+    g_launches.fetch_add(v->nodes);
     return FLD_OK;
 }
 
