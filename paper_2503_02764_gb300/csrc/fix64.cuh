@@ -32,13 +32,20 @@ __device__ __forceinline__ f32pair split_pos(double v) {
 
 // h + l as FP64 (h positive and normal, |l| below 64 units of h), l rounded to 2^-15 units of h:
 // 2^-39 of the value, which the residual correction takes to 2^-61 (1.5 * 2^23 rounds to the
-// integer).
+// integer). Where the sum leaves h's binade, the part beyond the power of two is in other units:
+// half as large below it, twice as large above. (Left as it is, that part would be off by half or
+// twice its size, up to 2^-23 of the value, and the quotient by 2^-46.)
 __device__ __forceinline__ double join_pos(float h, float l) {
     const unsigned u = __float_as_uint(h);
     const float per = __uint_as_float((277u << 23) - (u & 0x7F800000u));   // 1 / unit of h
     const int r = __float_as_int(__fmaf_rn(l * per, 32768.f, 12582912.f)) - 0x4B400000;
-    return __longlong_as_double(
-        (long long)(((unsigned long long)u + (896ull << 23)) << 29) + ((long long)r << 14));
+    const long long hb = (long long)(((unsigned long long)u + (896ull << 23)) << 29);
+    long long b = hb + ((long long)r << 14);
+    if ((b ^ hb) >> 52) {
+        const long long edge = (max(b, hb) >> 52) << 52;
+        b = b < edge ? 2 * b - edge : (b + edge) >> 1;
+    }
+    return __longlong_as_double(b);
 }
 
 __device__ __forceinline__ float rcp_fast(float a) {

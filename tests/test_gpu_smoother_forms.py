@@ -1,0 +1,53 @@
+"""The forms that smoothers 0 and 2 give a level (z-marching sweeps in 3D, tiles in 2D) against the
+out-of-place half sweeps of smoother 1, whose updates are the same: the iterate after one
+refinement step, cell by cell, whether or not the iteration would converge.
+
+Tolerance: the forms differ by the FP32 rounding of their relaxations (three units of 2^-24 each),
+which relaxations and transfers do not amplify in the max norm: with at most 60 relaxations on the
+way down and up the levels below 60 * 3 * 2^-24 = 1.1e-5 of the correction, and as much again for
+each of `inner` V-cycles."""
+import numpy as np
+import pytest
+
+from paper_2503_02764_gb300 import inputs as I
+from gpu_util import torch_cuda, library, dev, host
+
+pytestmark = pytest.mark.gpu
+
+P, N, D, M = (0, 0), (1, 1), (2, 2), (1, 2)
+CASES = [((24, 20, 32), (1 / 32, 1 / 20, 1 / 24), (P, P, D), 2e-4),
+         ((40, 36, 128), (1.0, 1.0, 1.0), (P, M, (2, 1)), 0.8),
+         ((18, 17, 68), (1.0, 0.9, 1.1), (D, N, P), 1.5), ((16, 16, 16), (1.0, 1.0, 1.0), (N, D, P), 30.0),
+         ((64, 66), (1.0, 0.8), (P, P), 40.0), ((33, 65), (1.0, 0.8), (N, D), 40.0),
+         ((17, 34), (1.0, 0.8), (D, P), 1.0), ((200, 280), (1.0, 0.8), (P, M), 40.0),
+         ((5, 40), (1.0, 0.8), (D, D), 40.0), ((40, 2), (1.0, 0.8), (P, P), 40.0)]
+OPTS = [dict(nu1=1, nu2=1), dict(nu1=2, nu2=2), dict(nu1=1, nu2=2), dict(nu1=2, nu2=1),
+        dict(nu1=1, nu2=0, inner=3), dict(nu1=0, nu2=3), dict(nu1=4, nu2=1, inner=2, prolong=1)]
+
+
+@pytest.mark.parametrize("opts", OPTS)
+@pytest.mark.parametrize("precision", [1, 2])
+@pytest.mark.parametrize("shape,h,bc,dt", CASES)
+def test_one_step_is_that_of_half_sweeps(shape, h, bc, dt, precision, opts):
+    torch = torch_cuda()
+    fld = library()
+    nd = len(shape)
+    rng = np.random.default_rng(sum(shape))
+    Dc = dev(torch, I.lognormal(rng, shape, 0.5, 4.0))
+    E = 1.0 + rng.uniform(0, 1, shape)
+    Eb = {(d, s): 1.0 + rng.uniform(0, 1, tuple(n for a, n in enumerate(shape) if a != nd - 1 - d))
+          for d in range(nd) for s in (0, 1) if bc[d][s] == 2}
+    packed = I.pack_dirichlet(shape, bc, Eb)
+    ebc = dev(torch, packed) if packed.size else None
+    hd = fld.Handle(shape, h, bc)
+    x = {}
+    for sm, graph in ((1, 0), (0, 0), (2, 1)):
+        hd.set_opts(precision=precision, tol=1e-14, max_cycles=1, smoother=sm, graph=graph, **opts)
+        xd = dev(torch, E)
+        hd.diffuse(dt, Dc, ebc, xd, raise_on_error=False)
+        x[sm] = host(xd)
+    size = np.max(np.abs(x[1] - E.ravel().reshape(x[1].shape)))
+    assert np.all(np.isfinite(x[1])) and size > 1e-3
+    assert np.max(np.abs(x[0] - x[1])) <= 1.1e-5 * opts.get("inner", 1) * size
+    assert np.array_equal(x[0], x[2])
+    hd.close()
