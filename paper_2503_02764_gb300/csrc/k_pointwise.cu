@@ -208,11 +208,13 @@ k_coupling(Lvl L, double3 inv12h, const double* __restrict__ E,
             }
             const double a = kr * Ec;
             double lam, lr, D, gn, q;          // lr = lambda R
+            bool far = false;                  // |grad E|^2 near the ends of the FP64 range
             if (mode != FLD_LIMITER_DIFFUSION && limiter_core<true>(a, g2, mode, one, true, gn, q, lam)) {
                 lr = gn * q;
                 D = c * Ec * q;
             } else {
                 gn = sqrt(g2);
+                far = abs((__double2hiint(g2) >> 20) - 1023) > 300 && gn > 0.0;
                 const double R = gn / a;
                 lam = mode == FLD_LIMITER_LP        ? (2.0 + R) / (6.0 + 3.0 * R + R * R)
                       : mode == FLD_LIMITER_MINERBO ? minerbo_lambda(R)
@@ -233,6 +235,22 @@ k_coupling(Lvl L, double3 inv12h, const double* __restrict__ E,
             if (fe) fe[p] = f;
             if (v && vfr) vfr[p] = vf;
             if (v && pt) {
+                // n n has no scale: where 1 / g^2, or g^2 times grad v, could leave the FP64 range,
+                // g is brought to order one first (at 2^-514, for instance, g^2 is subnormal). The
+                // empty statement keeps the FP64 instructions in their branch: they would be
+                // executed speculatively by every cell.
+                if (far) {
+                    asm volatile("");
+                    const int e = (__double2hiint(g2) >> 20) - 1023;
+                    const double sc =
+                        __hiloint2double((1023 + max(-511, min(-(e / 2), 511))) << 20, 0);
+                    g2 = 0.0;
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        g[d] *= sc;
+                        g2 = fma(g[d], g[d], g2);
+                    }
+                }
                 double gh[3], div = 0.0, S = 0.0;
                 const int cc[3] = {i, j, k};
 #pragma unroll
