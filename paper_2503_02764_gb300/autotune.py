@@ -2,7 +2,7 @@
 
 For the batched substep it times (threads per block, blocks per problem cluster,
 pre/post smoothing sweeps, FP32 V-cycles per refinement step); for a single grid
-(pre/post sweeps, smoother kind, V-cycles per refinement step). Each
+(pre/post sweeps, V-cycles per refinement step, and the smoother kinds asked for). Each
 candidate runs the real substep on a copy of the caller's fields; a candidate counts
 only if every problem reaches the tolerance. The fastest is cached in a JSON file keyed
 by the GPU name and a signature of the workload (shapes, boundary kinds), so later runs
@@ -38,8 +38,8 @@ def gpu_name():
 
 PRECISION_NAMES = {0: "fp64", 1: "mixed", 2: "mixed_df"}
 
-# options of a single grid when nothing is cached: V(2,2), in-place half sweeps, one FP32
-# V-cycle per refinement step
+# options of a single grid when nothing is cached: V(2,2), the fastest form of each level's
+# sweeps, one FP32 V-cycle per refinement step
 DEFAULT_GRID = {"nu1": 2, "nu2": 2, "smoother": 0, "inner": 1}
 
 
@@ -165,8 +165,9 @@ def tune_batch(problems, blocks=(256, 512, 1024), clusters=(1, 2, 4, 8),
 
 
 def tune_grid(problem, precision=2, sweeps=((2, 2), (1, 1), (2, 1), (1, 2), (3, 3)),
-              smoothers=(0, 2), inners=(1, 2, 3), tol=1e-10, store=True, reps=3, presteps=3):
-    """Time (nu1, nu2, smoother, inner) for one grid's full substep; return the best.
+              smoothers=(0,), inners=(1, 2, 3), tol=1e-10, store=True, reps=3, presteps=3):
+    """Time (nu1, nu2, smoother, inner) for one grid's full substep; return the best. Smoothers 0
+    and 2 run the same kernels, so that only one of them is a candidate.
 
     The fields are first advanced `presteps` substeps with the default options, so the
     candidates are timed on the state a running simulation meets after its first steps
