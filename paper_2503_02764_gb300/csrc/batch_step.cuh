@@ -525,9 +525,10 @@ __device__ void grp_exchange_df(const Grp<CS>& g, int n, const double* r, double
 // 512: 13.4 ms with a tile's memory reserved, 12.5 without; 512 lines: 2.07 and 1.72 ms).
 // Unclustered blocks of 256 threads run four an SM without tiles (64 registers): a problem of
 // 17^2 to 193^2 cells leaves most of a block waiting (600 of 65^2: 2.79 ms, three an SM 3.37,
-// two 3.30).
+// two 3.30). Blocks of 512 take 64 registers of themselves; asked for two an SM, ptxas orders the
+// loops for it, which costs 2 to 6 % (600 problems of 16^2: 1.09 ms, 1.03 without).
 template <int NT, int CS, bool TILED>
-__global__ void __launch_bounds__(NT, NT == 256 ? (CS == 1 && !TILED ? 4 : 2) : 1024 / NT)
+__global__ void __launch_bounds__(NT, NT == 256 ? (CS == 1 && !TILED ? 4 : 2) : 0)
 k_batch_step(const BProb* __restrict__ probs, const BDyn* __restrict__ dyn,
              const int* __restrict__ order, int nprob, int* __restrict__ queue, BatchParams prm,
              const double* __restrict__ rho, double* __restrict__ T, double* __restrict__ E,
