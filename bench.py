@@ -51,7 +51,9 @@ BYTES_PER_CELL = {
     "resid_upd": 32.0,        # x, e32, K32, r32 read; x + e, r32 written (r - A e in FP32)
     "resid_df": 40.0,         # x (hi, lo), e32, b (hi, lo), K (hi, lo) read; x (hi, lo), r32 written
     "rbhalf32": 10.0,         # one colour: the other colour's x and every K read (faces),
-    "rbhalf64": 28.0,         #   this colour's b read and x written (fp64: stored weights)
+                              #   this colour's b read and x written
+    "rbhalf64": 40.0,         # one colour: three weight arrays (every face meets it), the other
+                              #   colour's x, this colour's b and inverse diagonal read, x written
     "rbsweep32": 16.0,        # x, K, b read; x written (both colours in one pass)
     "rbsweep64": 32.0,
     "add_correction": 20.0,   # x, e32 read; x written

@@ -281,8 +281,8 @@ __device__ void grp_tiles(const Grp<CS>& g, const Lvl& F, const Lvl& C, T2Args a
     for (int t = g.rank; t < nt; t += CS) {
         const int y0 = (t / ntx) * ty;
         // the last tiles along y load the rows that are left (an even number: they restrict
-        // pairs), which is all of a coarse level (600 problems of 64^2, two blocks of 512 each:
-        // 4.42 ms with full tiles, 4.00 so)
+        // pairs), which is all of a coarse level (600 problems of 65^2, two blocks of 512 each:
+        // 6.5 ms with full tiles, 5.1 so)
         a.R = min(most, ((F.n[1] - y0 + 1) & ~1) + 2 * a.H);
         t2_tile<NT>(F, C, a, (t % ntx) * tx, y0, tile);
         __syncthreads();
@@ -522,7 +522,8 @@ __device__ void grp_exchange_df(const Grp<CS>& g, int n, const double* r, double
 
 // TILED: with the code and the shared memory of the tiles, for batches with a problem that
 // batch_tiled takes; the others keep their L1 and their registers (256 3D problems, blocks of
-// 512: 13.4 ms with a tile's memory reserved, 12.5 without; 512 lines: 2.07 and 1.72 ms).
+// 512, MIXED_DF: 12.8 ms with a tile's memory reserved, 12.5 without; 512 problems of 16 to 64
+// cells a side as half sweeps 1.72 and 1.69 ms).
 // Unclustered blocks of 256 threads run four an SM without tiles (64 registers): a problem of
 // 17^2 to 193^2 cells leaves most of a block waiting (600 of 65^2: 2.79 ms, three an SM 3.37,
 // two 3.30). Blocks of 512 take 64 registers of themselves; asked for two an SM, ptxas orders the

@@ -129,6 +129,15 @@ __device__ __forceinline__ df df_from_double(double v) {
 
 __device__ __forceinline__ double df_to_double(df x) { return (double)x.hi + (double)x.lo; }
 
+// The FP32 number nearest to an integer of magnitude up to 2^29, ties to even, from two exact
+// pieces and one FMA: the conversion instruction holds the FP64 pipe of this GPU for as
+// long as two FP64 instructions.
+__device__ __forceinline__ float f32_of_int(int v) {
+    const float hi = __uint_as_float(0x4B400000u + (unsigned)(v >> 14)) - 12582912.f;
+    const float lo = __uint_as_float(0x4B400000u + (unsigned)(v & 0x3FFF)) - 12582912.f;
+    return __fmaf_rn(hi, 16384.f, lo);
+}
+
 // The same two conversions in integer arithmetic (FP64 instructions issue at 1/58 of the
 // FP32 rate here, and a conversion costs about two of them), bit-identical to the FP64
 // forms above; each returns false outside its window and the caller then uses those.
@@ -136,16 +145,7 @@ __device__ __forceinline__ double df_to_double(df x) { return (double)x.hi + (do
 // split: v * 2^k2 -> (RN32, RN32 of the remainder), for 2^-48 <= |v 2^k2| < 2^80. hi is
 // the double's significand rounded to 24 bits (ties to even, a carry moving it to the next
 // binade); the remainder v - hi is an integer number of the double's ulps below 2^29,
-// rounded to 24 bits by the int -> float conversion and scaled through its exponent field.
-//
-// f32_of_int: the FP32 number nearest to a 32-bit integer, ties to even, from two
-// exact pieces and one FMA: the conversion instruction holds the FP64 pipe of this GPU for as
-// long as two FP64 instructions.
-__device__ __forceinline__ float f32_of_int(int v) {
-    const float hi = __uint_as_float(0x4B400000u + (unsigned)(v >> 14)) - 12582912.f;
-    const float lo = __uint_as_float(0x4B400000u + (unsigned)(v & 0x3FFF)) - 12582912.f;
-    return __fmaf_rn(hi, 16384.f, lo);
-}
+// rounded to 24 bits by f32_of_int and scaled through its exponent field.
 __device__ __forceinline__ bool df_split_i(double v, int k2, df& out) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     const unsigned sgn = (unsigned)(b >> 63);

@@ -1,10 +1,10 @@
 // FP64 V-cycle kernels of 2D and 3D levels on stored coefficients.
 //
-// FP64 instructions bound these kernels, not memory: this GPU issues 0.6 T of them a second,
-// 64 times fewer than FP32 ones. Evaluating the face coefficients from K in every half
-// sweep took about 40 FP64 instructions per updated cell (six sums, six weightings, the diagonal
-// and a division): 651 us per half sweep of a 256^3 level. The coefficients do not change
-// during a solve, so they are formed once per level and solve:
+// FP64 instructions bound these kernels, not memory: this GPU issues 0.5 T of them a second
+// (19.2 cycles of an SM a warp), some 75 times fewer than FP32 ones. Evaluating the face
+// coefficients from K in every half sweep took about 40 FP64 instructions per updated cell (six
+// sums, six weightings, the diagonal and a division): 651 us per half sweep of a 256^3 level. The
+// coefficients do not change during a solve, so they are formed once per level and solve:
 //   wx, wy, wz  the weight mean(K_p, K_q) w_d of the face towards the lower neighbour along
 //               each axis (the wrapped face for the first cell of a periodic axis; 0 at walls),
 //   inv         1 / (1 + the six weights + 2 K w_d per Dirichlet face),

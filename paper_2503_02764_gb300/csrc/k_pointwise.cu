@@ -8,9 +8,10 @@ namespace fld {
 
 // ----------------------------------------------------------------- exchange
 // Backward Euler on de/dt = +qdot, dE/dt = -qdot with qdot = c kappa rho (E - a_r T^4)
-// (Eqs. heating, qdot). Eliminating E' leaves, per cell,
-//   f(T) = alpha T + beta T^4 - q = 0,  alpha = rho c_v, beta = a_r chi/(1+chi),
-//   q = e + chi E/(1+chi),  chi = dt c kappa rho,
+// (Eqs. heating, qdot). Eliminating E' and multiplying by 1 + chi, chi = dt c kappa rho, leaves,
+// per cell,
+//   f(T) = alpha T + beta T^4 - q = 0,  alpha = rho c_v (1 + chi), beta = a_r chi,
+//   q = alpha T^n + chi E,
 // increasing and convex for T > 0 with f(0) < 0: one positive root, bounded above by
 // min(q/alpha, (q/beta)^(1/4)), from where Newton decreases monotonically to it.
 //
