@@ -41,7 +41,8 @@ __device__ __forceinline__ double join_pos(float h, float l) {
     const int r = __float_as_int(__fmaf_rn(l * per, 32768.f, 12582912.f)) - 0x4B400000;
     const long long hb = (long long)(((unsigned long long)u + (896ull << 23)) << 29);
     long long b = hb + ((long long)r << 14);
-    if ((b ^ hb) >> 52) {
+    if (__builtin_expect((((int)(b >> 32) ^ (int)(hb >> 32)) & 0x7FF00000) != 0, 0)) {
+        asm volatile("");              // a branch: not executed by every cell
         const long long edge = (max(b, hb) >> 52) << 52;
         b = b < edge ? 2 * b - edge : (b + edge) >> 1;
     }
